@@ -17,11 +17,10 @@
 // convention of k_hetrd), so T = Q^H H_F Q is real and Q = prod_j prod_s H(j, s).
 //
 // Pipelining: sweep j+1 may run its step s once sweep j has finished step s+1 (their later
-// steps touch disjoint entries), so several sweeps are in flight at once.  One CTA per system;
-// NG groups of G threads each take every NG-th sweep, publish their progress in shared memory and
-// wait (bounded) for their predecessor's.  A step stages its two b x b blocks in the group's
-// shared memory; the band itself stays in the dense matrix's lower triangle (global memory,
-// L2-resident: about n x 2b entries are ever touched).
+// steps touch disjoint entries), so several sweeps are in flight at once, each with a group of
+// threads of its own that publishes its progress and waits (bounded) for its predecessor's.  The
+// band itself stays in the dense matrix's lower triangle (global memory, L2-resident: about n x 2b
+// entries are ever touched).
 //
 // Back-transform: Z = Q Y.  Reflectors of one sweep touch disjoint rows, and H(j', s') must
 // precede H(j, s) only if j' > j and s' in {s-1, s}, so the order "s ascending, j descending"
@@ -45,45 +44,130 @@ int64_t mmf_sbr_store_elems(int n, int b) { return sbr_nref(n, b) * (b + 1); }
 // 256 so that the blocks' 16-byte complex elements stay aligned
 __host__ __device__ constexpr int sbr_hdr(int ng) { return (8 * ng + 16 + 255) / 256 * 256; }
 
+// A vector entry in shared memory as the multiplier of packed products: (x, x), (y, y).  With it
+// acc1 += a (x, x) and acc2 += a (y, y) are two packed FP32 instructions, and
+// a v = (acc1.x - acc2.y, acc1.y + acc2.x), conj(v) a = (acc1.x + acc2.y, acc1.y - acc2.x).  The
+// FP64 path keeps plain entries.
+template <class C> struct SbrDup;
+template <> struct SbrDup<float2> {
+    typedef float4 T;
+    static __device__ __forceinline__ T of(float2 v) { return make_float4(v.x, v.x, v.y, v.y); }
+    static __device__ __forceinline__ float2 val(T t) { return make_float2(t.x, t.z); }
+};
+template <> struct SbrDup<double2> {
+    typedef double2 T;
+    static __device__ __forceinline__ T of(double2 v) { return v; }
+    static __device__ __forceinline__ double2 val(T t) { return t; }
+};
+// running sum of a v and of conj(v) a over entries v
+template <class C> struct SbrAcc;
+template <> struct SbrAcc<float2> {
+    float2 p, q;
+    __device__ __forceinline__ SbrAcc() : p(make_float2(0.f, 0.f)), q(make_float2(0.f, 0.f)) {}
+    __device__ __forceinline__ void add(float2 a, float4 v) {
+        p = __ffma2_rn(a, make_float2(v.x, v.y), p);
+        q = __ffma2_rn(a, make_float2(v.z, v.w), q);
+    }
+    __device__ __forceinline__ void addc(float2 a, float4 v) { add(a, v); }
+    __device__ __forceinline__ float2 mul() const { return make_float2(p.x - q.y, p.y + q.x); }
+    __device__ __forceinline__ float2 mulc() const { return make_float2(p.x + q.y, p.y - q.x); }
+};
+template <> struct SbrAcc<double2> {
+    double2 p;
+    __device__ __forceinline__ SbrAcc() : p(make_double2(0.0, 0.0)) {}
+    __device__ __forceinline__ void add(double2 a, double2 v) { p = p + a * v; }
+    __device__ __forceinline__ void addc(double2 a, double2 v) { p = p + cmulc(v, a); }
+    __device__ __forceinline__ double2 mul() const { return p; }
+    __device__ __forceinline__ double2 mulc() const { return p; }
+};
+// a - f conj(v) (rank-1 update by a row of conjugated entries) and a - f v
+__device__ __forceinline__ float2 sbr_sub_conj(float2 a, float2 f, float4 v) {
+    a = __ffma2_rn(make_float2(-f.x, -f.y), make_float2(v.x, v.y), a);
+    return __ffma2_rn(make_float2(-f.y, f.x), make_float2(v.z, v.w), a);
+}
+__device__ __forceinline__ double2 sbr_sub_conj(double2 a, double2 f, double2 v) { return a - cmulc(v, f); }
+__device__ __forceinline__ float2 sbr_sub(float2 a, float2 f, float4 v) {
+    a = __ffma2_rn(make_float2(-f.x, -f.y), make_float2(v.x, v.y), a);
+    return __ffma2_rn(make_float2(f.y, -f.x), make_float2(v.z, v.w), a);
+}
+__device__ __forceinline__ double2 sbr_sub(double2 a, double2 f, double2 v) { return a - f * v; }
+
+// Shared memory of one group.  B and D: the step's two blocks, column-major with a padded column
+// (LD even: two rows of a column are one aligned 16-byte read, and consecutive columns fall in
+// other banks).
 template <class C, int BMAX, int P>
-struct SbrGroup {
-    C B[BMAX][BMAX + 1];
-    C Dm[BMAX][BMAX + 1];
-    C v[2][BMAX];   // current and previous reflector
-    C y[BMAX], w[BMAX];
-    C red[P][BMAX];
-    C tau[2];
-    double rs[32];
-    int stop;  // the group's copy of the abort flag, taken by its first thread after each wait
-    int pad[3];
+struct __align__(16) SbrGroup {
+    static constexpr int LD = BMAX + 2;
+    typedef typename SbrDup<C>::T Dup;
+    Dup v[2][BMAX];      // current and previous reflector
+    Dup wu[BMAX], wd[BMAX];
+    C B[BMAX * LD];
+    C D[BMAX * LD];
+    C red[3][P][BMAX];   // partial sums: B v_p, v^H B, D v
+    C c0[BMAX];          // B(:, 0)
+    C ty[BMAX];
+    C beta[2];
 };
 
-// Asynchronous copy of one complex element global -> shared (8 or 16 bytes); ok = false fills
-// zeros without reading (the source address given is then any valid one).
-template <class C>
-__device__ __forceinline__ void cp_elem(C* sdst, const C* gsrc, bool ok) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(sdst);
-    if (sizeof(C) == 16)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gsrc), "r"(ok ? 16 : 0) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(gsrc), "r"(ok ? 8 : 0) : "memory");
-}
-// Load of one complex element from L2, bypassing L1: the two CTAs of a cluster run on different
-// SMs, whose L1 caches are not coherent, so band data written by one must not be read by the other
-// from a stale L1 line.
-__device__ __forceinline__ float2 ld_cg(const float2* p) {
+// Predicated load (zero where !ok) and store of one complex element, without a branch around each.
+// CG reads L2 only: the CTAs of a cluster run on different SMs, whose L1 caches are not coherent, so
+// band data written by one must not be read by another from a stale L1 line.
+template <bool CG>
+__device__ __forceinline__ float2 ld_if(const float2* p, bool ok) {
     float2 r;
-    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    if (CG)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f32 %0, 0f00000000;\n\t"
+                     "mov.f32 %1, 0f00000000;\n\t@p ld.global.cg.v2.f32 {%0, %1}, [%2];\n\t}"
+                     : "=&f"(r.x), "=&f"(r.y) : "l"(p), "r"((int)ok) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f32 %0, 0f00000000;\n\t"
+                     "mov.f32 %1, 0f00000000;\n\t@p ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
+                     : "=&f"(r.x), "=&f"(r.y) : "l"(p), "r"((int)ok) : "memory");
     return r;
 }
-__device__ __forceinline__ double2 ld_cg(const double2* p) {
+template <bool CG>
+__device__ __forceinline__ double2 ld_if(const double2* p, bool ok) {
     double2 r;
-    asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "l"(p));
+    if (CG)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f64 %0, 0d0000000000000000;\n\t"
+                     "mov.f64 %1, 0d0000000000000000;\n\t@p ld.global.cg.v2.f64 {%0, %1}, [%2];\n\t}"
+                     : "=&d"(r.x), "=&d"(r.y) : "l"(p), "r"((int)ok) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f64 %0, 0d0000000000000000;\n\t"
+                     "mov.f64 %1, 0d0000000000000000;\n\t@p ld.global.v2.f64 {%0, %1}, [%2];\n\t}"
+                     : "=&d"(r.x), "=&d"(r.y) : "l"(p), "r"((int)ok) : "memory");
     return r;
 }
-__device__ __forceinline__ void cp_wait_all() {
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+__device__ __forceinline__ void st_if(float2* p, float2 v, bool ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p st.global.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(p),
+                 "f"(v.x), "f"(v.y), "r"((int)ok)
+                 : "memory");
+}
+__device__ __forceinline__ void st_if(double2* p, double2 v, bool ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p st.global.v2.f64 [%0], {%1, %2};\n\t}" ::"l"(p),
+                 "d"(v.x), "d"(v.y), "r"((int)ok)
+                 : "memory");
+}
+
+// progress key of a group, in its CTA's shared memory (addressed as shared::cluster)
+__device__ __forceinline__ long long key_load(uint32_t a) {
+    long long v;
+    asm volatile("ld.acquire.cluster.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ int flag_load(uint32_t a) {
+    int v;
+    asm volatile("ld.relaxed.cluster.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void key_store(uint32_t a, long long v) {
+    asm volatile("st.release.cluster.shared::cluster.b64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+// address of this CTA's shared memory location in the CTA of the given rank
+__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
 }
 
 template <int G>
@@ -95,18 +179,24 @@ __device__ __forceinline__ void gbar(int g) {
     }
 }
 
-// sum over the G threads of the group (every thread gets the result)
-template <int G, class R>
-__device__ __forceinline__ R group_sum(R v, double* rs, int tid, int g) {
-    v = warp_sum(v);
-    if (G == 32) return v;
-    if ((tid & 31) == 0) rs[tid >> 5] = (double)v;
-    gbar<G>(g);
-    double s = 0.0;
+// sum over the lanes that hold different entries of a vector of BMAX (all 32, or BMAX of them when
+// the vector is repeated over the warp); every lane gets the result
+template <int BMAX, class R>
+__device__ __forceinline__ R lane_sum(R v) {
 #pragma unroll
-    for (int k = 0; k < G / 32; ++k) s += rs[k];
-    gbar<G>(g);
-    return (R)s;
+    for (int o = BMAX < 32 ? BMAX / 2 : 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// two consecutive complex entries of a column
+__device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    a = make_float2(t.x, t.y);
+    b = make_float2(t.z, t.w);
+}
+__device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b) {
+    a = p[0];
+    b = p[1];
 }
 
 template <class R> __device__ __forceinline__ R rsqrt_of(R x);
@@ -131,76 +221,48 @@ __device__ __forceinline__ void make_reflector(C alpha, R xn2, C& tau, R& beta, 
     scale = mk(den.x / dd, -den.y / dd);
 }
 
-// Two-sided update A <- H^H A H of the l x l Hermitian block held (both triangles) in Dm, with
-// H = I - tau v v^H: y = A v, w = tau y - |tau|^2 (v^H y) / 2 v, A -= v w^H + w v^H; the lower
-// triangle is written to global memory at Hg (column-major, ld) from row/column r.
-template <class R, class C, int BMAX, int G, int P>
-__device__ __forceinline__ void sbr_two_sided(SbrGroup<C, BMAX, P>& S, const C* v, C tau, int l, C* __restrict__ Hg,
-                                              int ld, int r, int tid, int g, double* dout) {
-    const int i = tid % BMAX, p = tid / BMAX;
-    C acc = mk(R(0), R(0)), acc1 = acc;  // two partial sums: independent FMA chains
-#pragma unroll
-    for (int q = 0; q < BMAX / P; q += 2) {
-        acc = acc + S.Dm[i][p + q * P] * v[p + q * P];
-        acc1 = acc1 + S.Dm[i][p + (q + 1) * P] * v[p + (q + 1) * P];
-    }
-    S.red[p][i] = acc + acc1;
-    gbar<G>(g);
-    R a_part = R(0);
-    if (tid < BMAX) {
-        C yy = S.red[0][tid];
-#pragma unroll
-        for (int q = 1; q < P; ++q) yy = yy + S.red[q][tid];
-        S.y[tid] = yy;
-        const C vv = v[tid];
-        a_part = vv.x * yy.x + vv.y * yy.y;  // Re(conj(v) y)
-    }
-    const R a = group_sum<G, R>(a_part, S.rs, tid, g);
-    const R t2 = R(0.5) * (tau.x * tau.x + tau.y * tau.y) * a;
-    if (tid < BMAX) S.w[tid] = tau * S.y[tid] - t2 * v[tid];
-    gbar<G>(g);
-    // lower triangle, column by column (rows i >= k contiguous in global memory)
-    const C vi = v[i], wi = S.w[i];
-#pragma unroll
-    for (int q = 0; q < BMAX / P; ++q) {
-        const int k = p + q * P;
-        if (i >= k && i < l) {
-            const C vk = v[k], wk = S.w[k];
-            C a0 = S.Dm[i][k];
-            a0 = a0 - cmulc(wk, vi) - cmulc(vk, wi);  // v_i conj(w_k) + w_i conj(v_k)
-            if (i == k) {
-                a0.y = R(0);
-                if (dout && i == 0) *dout = (double)a0.x;
-            }
-            Hg[(r + k) * ld + r + i] = a0;
-        }
-    }
-}
-
-// CL = 1: one CTA per system.  CL = 2: a cluster of two CTAs (two SMs) per system, the sweeps
-// dealt round-robin over both CTAs' groups; a group reads its predecessor's progress key from the
-// partner's shared memory (distributed shared memory), the band is read from L2 only (ld.cg), and
-// progress is published after a GPU-scope fence.
-template <class R, int BMAX, int G, int NG, int CL>
-__global__ void __launch_bounds__(G* NG) k_sbr_chase(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
-                                                    typename Cx<R>::T* __restrict__ Hbase,
-                                                    typename Cx<R>::T* __restrict__ store_base,
-                                                    double* __restrict__ dvec, double* __restrict__ evec,
-                                                    int* __restrict__ status) {
+// One group of G = BMAX P threads per sweep: thread (i, p) keeps row i, columns p EL .. p EL + EL - 1
+// of the step's two blocks B = A(R_s, R_{s-1}) and D = A(R_s, R_s) (lower triangle) in registers,
+// from its loads to its stores; a copy in shared memory serves the sums down the columns.  A step is
+//   load | y = B v_p (partial sums) | x = B(:,0) - tau_p y gives v, tau, beta | u = v^H B and D v
+//   (rows from registers, columns from shared memory) | w vectors | rank-2 updates, store
+// with five group barriers; one warp computes the vectors.
+//
+// What bounds it: the critical path of about 2n steps of one sweep after another (a sweep starts two
+// steps behind its predecessor), so the latency of a step; on the FP64 path the 2 FP64 FMAs per clock
+// of an SM (about 25 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
+// CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
+// b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
+// kernel): one system in FP32 36.2 -> 15.5 ms, 64 systems 37.4 -> 24.3 ms; eight systems in FP64
+// 455 -> 147 ms.
+//
+// CL = 1: one CTA per system.  CL > 1: a cluster of CL CTAs per system, the sweeps dealt round-robin
+// over all groups; a group reads its predecessor's progress key from that CTA's shared memory
+// (distributed shared memory; the key is stored with release and read with acquire semantics, each
+// warp polling for itself), and the band is read from L2 only (ld.cg).  A wait that gives up marks
+// the system and makes every group run on without waiting (its results are void, every access stays
+// in bounds), so that the group's warps pass the same barriers.
+template <class R, int BMAX, int P, int NG, int CL>
+__global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __restrict__ descs,
+                                                          const int* __restrict__ idx,
+                                                          typename Cx<R>::T* __restrict__ Hbase,
+                                                          typename Cx<R>::T* __restrict__ store_base,
+                                                          double* __restrict__ dvec, double* __restrict__ evec,
+                                                          int* __restrict__ status) {
     typedef typename Cx<R>::T C;
-    constexpr int P = G / BMAX;
-    static_assert(P * BMAX == G && P >= 1, "group size is a multiple of BMAX");
-    constexpr int NGT = CL * NG;                          // groups per system
-    constexpr int LCH = (BMAX / P) < 16 ? (BMAX / P) : 16;  // register-staged loads per batch (CL > 1)
-    static_assert((BMAX / P) % LCH == 0, "load batches divide the block");
+    typedef SbrGroup<C, BMAX, P> Grp;
+    typedef SbrDup<C> DupC;
+    constexpr int G = BMAX * P, EL = BMAX / P, LD = Grp::LD;
+    constexpr int SL = BMAX >= 32 ? BMAX / 32 : 1;  // entries of a vector per lane
+    constexpr bool F64 = sizeof(R) == 8;            // FP64 units are scarce: skip padding
+    constexpr int NGT = CL * NG;                    // groups per system
+    static_assert(G % 32 == 0 && EL * P == BMAX && EL % 2 == 0, "group shape");
     extern __shared__ __align__(16) unsigned char sbr_smem[];
-    volatile long long* key = reinterpret_cast<volatile long long*>(sbr_smem);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(sbr_smem + 8 * NG);
-    SbrGroup<C, BMAX, P>* groups = reinterpret_cast<SbrGroup<C, BMAX, P>*>(sbr_smem + sbr_hdr(NG));
+    long long* key = reinterpret_cast<long long*>(sbr_smem);
+    int* abort_flag = reinterpret_cast<int*>(sbr_smem + 8 * NG);
+    Grp* groups = reinterpret_cast<Grp*>(sbr_smem + sbr_hdr(NG));
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = CL > 1 ? (int)cluster.block_rank() : 0;
-    volatile int* abort_peer = abort_flag;
-    if (CL > 1) abort_peer = cluster.map_shared_rank(const_cast<int*>(abort_flag), rank ^ 1);
 
     const int sid = idx[blockIdx.x / CL];
     const MmfDesc d = descs[sid];
@@ -213,220 +275,245 @@ __global__ void __launch_bounds__(G* NG) k_sbr_chase(const MmfDesc* __restrict__
     double* dd = dvec + d.vec_off;
     double* ee = evec + d.vec_off;
     const int g = threadIdx.x / G, tid = threadIdx.x % G;
+    const int lane = tid & 31, warp = tid >> 5;
     const int gg = rank * NG + g;  // the group's number within the system
-    SbrGroup<C, BMAX, P>& S = groups[g];
+    Grp& S = groups[g];
     const long long KK = sbr_passes(n, b) + 3;
-    // the predecessor sweep's group and its progress key (possibly in the partner CTA)
+    // the predecessor sweep's group, its progress key and its CTA's abort flag
     const int ggp = (gg + NGT - 1) % NGT;
-    volatile long long* pkey = key + (ggp % NG);
-    if (CL > 1 && ggp / NG != rank)
-        pkey = cluster.map_shared_rank(const_cast<long long*>(key), ggp / NG) + (ggp % NG);
+    const uint32_t pkey = map_rank(key + ggp % NG, ggp / NG), pabort = map_rank(abort_flag, ggp / NG);
+    const uint32_t mykey = map_rank(key + g, rank);
 
     if (threadIdx.x < NG) key[threadIdx.x] = -1;
     if (threadIdx.x == 0) *abort_flag = 0;
     if (CL > 1) cluster.sync(); else __syncthreads();
     if (threadIdx.x == 0 && rank == 0) dd[0] = (double)Hg[0].x;
 
+    const C zero = mk(R(0), R(0));
     const int i = tid % BMAX, p = tid / BMAX;
+    const int k0 = p * EL;                     // this thread's columns (and rows, in the column sums)
+    const int i0 = BMAX >= 32 ? (i & ~31) : 0; // the warp's first row
+    const bool low = k0 + EL - 1 > i0, row = k0 <= i0 + 31;  // the warp's share of D: column / row sums
     int cur = 0;  // buffer of the current reflector in S.v
     bool stopped = false;
-    for (int j = gg; j <= n - 2 && !stopped; j += NGT) {
+    C tau = zero, taup = zero;
+    for (int j = gg; j <= n - 2; j += NGT) {
         const int nsteps = (n - 2 - j) / b + 1;
         for (int s = 0; s < nsteps; ++s) {
             // wait until sweep j-1 has finished step s+1 (or all of its steps)
-            if (j > 0) {
-                if (tid == 0) {
+            if (j > 0 && !stopped) {
+                if (lane == 0) {
                     const long long need = (long long)(j - 1) * KK + (s + 2 < KK - 1 ? s + 2 : KK - 1);
                     int it = 0;
-                    while (*pkey < need && !*abort_flag && !*abort_peer) {
-                        if (++it > SBR_WAIT_LIMIT) {
-                            *abort_flag = 1;
+                    while (key_load(pkey) < need) {
+                        const int gave_up = ++it > SBR_WAIT_LIMIT;
+                        if (gave_up || flag_load(pabort) || *(volatile int*)abort_flag) {
+                            *(volatile int*)abort_flag = 1;  // the successors' CTAs see it too
                             status[sid] = MMF_ST_NOCONV;
+                            stopped = true;
                             break;
                         }
-                        __nanosleep(64);
+                        __nanosleep(32);
                     }
-                    if (CL > 1) __threadfence(); else __threadfence_block();
-                    S.stop = *abort_flag || *abort_peer;
                 }
-                gbar<G>(g);
-                if (S.stop) {  // the whole group leaves together
-                    stopped = true;
-                    break;
-                }
+                stopped = __shfl_sync(0xffffffffu, stopped, 0);
             }
-            const int r = j + 1 + s * b;
+            const int r = j + 1 + s * b, rp = r - b;
             const int l = min(b, n - r);
-            C* vc = S.v[cur];
-            const C* vp = S.v[cur ^ 1];
-            C tau;
-            if (s == 0) {
-                // column j below the diagonal and the diagonal block, lower triangle
-                // all of the step's loads in flight at once (asynchronous copies, zero-filled
-                // outside the l x l block)
-                if (CL == 1) {
-                    if (tid < BMAX) cp_elem(&vc[tid], Hg + j * ldi + r + (tid < l ? tid : 0), tid < l);
+            // (a) the step's entries: all loads in flight together, zeros outside the blocks
+            C B[EL], D[EL], x[SL];
+            {
+                const C* h = Hg + (r + k0) * ldi + r + i;
 #pragma unroll
-                    for (int q = 0; q < BMAX / P; ++q) {
-                        const int k = p + q * P;
-                        const bool ok = i < l && k < l && i >= k;
-                        cp_elem(&S.Dm[i][k], Hg + (ok ? (r + k) * ldi + r + i : 0), ok);
-                    }
-                    cp_wait_all();
-                } else {
-                    const C z0 = mk(R(0), R(0));
-                    if (tid < BMAX) vc[tid] = tid < l ? ld_cg(Hg + j * ldi + r + tid) : z0;
+                for (int q = 0; q < EL; ++q)
+                    D[q] = ld_if<(CL > 1)>(h + q * ldi, i < l && i >= k0 + q);
+            }
+            if (s > 0) {
+                const C* h = Hg + (rp + k0) * ldi + r + i;
 #pragma unroll
-                    for (int q0 = 0; q0 < BMAX / P; q0 += LCH) {
-                        C rd[LCH];
+                for (int q = 0; q < EL; ++q)
+                    B[q] = ld_if<(CL > 1)>(h + q * ldi, i < l && k0 + q < b);
+            } else if (warp == 0) {
 #pragma unroll
-                        for (int u = 0; u < LCH; ++u) {
-                            const int k = p + (q0 + u) * P;
-                            rd[u] = (i < l && k < l && i >= k) ? ld_cg(Hg + (r + k) * ldi + r + i) : z0;
-                        }
-#pragma unroll
-                        for (int u = 0; u < LCH; ++u) S.Dm[i][p + (q0 + u) * P] = rd[u];
-                    }
-                }
-                gbar<G>(g);
-#pragma unroll
-                for (int q = 0; q < BMAX / P; ++q) {
-                    const int k = p + q * P;
-                    if (i < k) S.Dm[i][k] = conj(S.Dm[k][i]);
-                }
-                const C alpha = vc[0];
-                const R xn2 = group_sum<G, R>((tid >= 1 && tid < l) ? abs2(vc[tid]) : R(0), S.rs, tid, g);
-                R beta;
-                C scale;
-                make_reflector<R, C>(alpha, xn2, tau, beta, scale);
-                if (tid < BMAX) {
-                    const C x = vc[tid];
-                    vc[tid] = tid == 0 ? mk(R(1), R(0)) : ((tid < l) ? x * scale : mk(R(0), R(0)));
-                    if (tid < l) Hg[j * ldi + r + tid] = tid == 0 ? mk(beta, R(0)) : mk(R(0), R(0));
-                }
-                if (tid == 0) {
-                    ee[j] = (double)beta;
-                    S.tau[cur] = tau;
-                }
-            } else {
-                const int rp = r - b;
-                const int lp = min(b, n - rp);
-                const C taup = S.tau[cur ^ 1];
-                if (CL == 1) {
-#pragma unroll
-                    for (int q = 0; q < BMAX / P; ++q) {
-                        const int k = p + q * P;
-                        const bool okb = i < l && k < lp, okd = i < l && k < l && i >= k;
-                        cp_elem(&S.B[i][k], Hg + (okb ? (rp + k) * ldi + r + i : 0), okb);
-                        cp_elem(&S.Dm[i][k], Hg + (okd ? (r + k) * ldi + r + i : 0), okd);
-                    }
-                    cp_wait_all();
-                } else {
-                    const C z0 = mk(R(0), R(0));
-#pragma unroll
-                    for (int q0 = 0; q0 < BMAX / P; q0 += LCH) {
-                        C rb[LCH], rd[LCH];
-#pragma unroll
-                        for (int u = 0; u < LCH; ++u) {
-                            const int k = p + (q0 + u) * P;
-                            rb[u] = (i < l && k < lp) ? ld_cg(Hg + (rp + k) * ldi + r + i) : z0;
-                            rd[u] = (i < l && k < l && i >= k) ? ld_cg(Hg + (r + k) * ldi + r + i) : z0;
-                        }
-#pragma unroll
-                        for (int u = 0; u < LCH; ++u) {
-                            S.B[i][p + (q0 + u) * P] = rb[u];
-                            S.Dm[i][p + (q0 + u) * P] = rd[u];
-                        }
-                    }
-                }
-                gbar<G>(g);
-#pragma unroll
-                for (int q = 0; q < BMAX / P; ++q) {
-                    const int k = p + q * P;
-                    if (i < k) S.Dm[i][k] = conj(S.Dm[k][i]);
-                }
-                // The previous reflector from the right and the new one from the left, as one rank-2
-                // update: with C1 = B H(j,s-1) = B - tau_p y v_p^H (y = B v_p), x = C1(:, 0) gives
-                // H(j,s); then H^H C1 = B - tau_p y v_p^H - conj(tau) v r with
-                // r_k = (v^H B)_k - tau_p (v^H y) conj(v_p,k).
-                C acc = mk(R(0), R(0)), acc1 = acc;
-#pragma unroll
-                for (int q = 0; q < BMAX / P; q += 2) {
-                    acc = acc + S.B[i][p + q * P] * vp[p + q * P];
-                    acc1 = acc1 + S.B[i][p + (q + 1) * P] * vp[p + (q + 1) * P];
-                }
-                S.red[p][i] = acc + acc1;
-                gbar<G>(g);
-                if (tid < BMAX) {
-                    C yy = S.red[0][tid];
-#pragma unroll
-                    for (int q = 1; q < P; ++q) yy = yy + S.red[q][tid];
-                    const C ty = taup * yy;
-                    S.y[tid] = ty;                      // tau_p y
-                    S.w[tid] = S.B[tid][0] - ty;        // x = C1(:, 0)   (v_p[0] = 1)
-                }
-                gbar<G>(g);
-                const C alpha = S.w[0];
-                const R xn2 = group_sum<G, R>((tid >= 1 && tid < l) ? abs2(S.w[tid]) : R(0), S.rs, tid, g);
-                R beta;
-                C scale;
-                make_reflector<R, C>(alpha, xn2, tau, beta, scale);
-                if (tid < BMAX) {
-                    const C x = S.w[tid];
-                    vc[tid] = tid == 0 ? mk(R(1), R(0)) : ((tid < l) ? x * scale : mk(R(0), R(0)));
-                }
-                if (tid == 0) S.tau[cur] = tau;
-                gbar<G>(g);
-                // u_k = sum_i conj(v_i) B(i, k) and gamma = v^H (tau_p y)
-                {
-                    const int kc = tid % BMAX, pc = tid / BMAX;
-                    C z = mk(R(0), R(0)), z1 = z;
-#pragma unroll
-                    for (int q = 0; q < BMAX / P; q += 2) {
-                        z = z + cmulc(vc[pc + q * P], S.B[pc + q * P][kc]);
-                        z1 = z1 + cmulc(vc[pc + (q + 1) * P], S.B[pc + (q + 1) * P][kc]);
-                    }
-                    S.red[pc][kc] = z + z1;
-                }
-                gbar<G>(g);
-                const R gre = group_sum<G, R>(tid < BMAX ? vc[tid].x * S.y[tid].x + vc[tid].y * S.y[tid].y : R(0),
-                                              S.rs, tid, g);
-                const R gim = group_sum<G, R>(tid < BMAX ? vc[tid].x * S.y[tid].y - vc[tid].y * S.y[tid].x : R(0),
-                                              S.rs, tid, g);
-                if (tid < BMAX) {
-                    C u = S.red[0][tid];
-#pragma unroll
-                    for (int q = 1; q < P; ++q) u = u + S.red[q][tid];
-                    // r_k = u_k - gamma conj(v_p,k), gamma = v^H (tau_p y); stored conj(tau) r_k
-                    const C rk = u - mk(gre, gim) * conj(vp[tid]);
-                    S.w[tid] = conj(tau) * rk;
-                }
-                gbar<G>(g);
-                {
-                    const C ty = S.y[i], vi = vc[i];
-#pragma unroll
-                    for (int q = 0; q < BMAX / P; ++q) {
-                        const int k = p + q * P;
-                        C bk = S.B[i][k] - ty * conj(vp[k]) - vi * S.w[k];
-                        if (k == 0) bk = i == 0 ? mk(beta, R(0)) : mk(R(0), R(0));
-                        if (i < l && k < lp) Hg[(rp + k) * ldi + r + i] = bk;
-                    }
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    x[u] = ld_if<(CL > 1)>(Hg + j * ldi + r + e, e < l);
                 }
             }
-            // store the reflector for the back-transform, marked evict-first: the store is written
-            // once and read only after the chase, and L2 should keep the band's lines instead
-            if (tid < b) __stcs(&V[(sbr_off(n, b, s) + j) * b + tid], vc[tid]);
-            if (tid == 0) __stcs(&T[sbr_off(n, b, s) + j], tau);
+#pragma unroll
+            for (int q = 0; q < EL; ++q) S.D[(k0 + q) * LD + i] = i == k0 + q ? zero : D[q];
+            if (s > 0) {
+                // y = B v_p over this thread's columns
+                const auto* vp = S.v[cur ^ 1] + k0;
+                SbrAcc<C> a0, a1;  // two partial sums: independent FMA chains
+#pragma unroll
+                for (int q = 0; q < EL; q += 2) {
+                    S.B[(k0 + q) * LD + i] = B[q];
+                    S.B[(k0 + q + 1) * LD + i] = B[q + 1];
+                    if (!F64 || k0 + q < b) {
+                        a0.add(B[q], vp[q]);
+                        a1.add(B[q + 1], vp[q + 1]);
+                    }
+                }
+                S.red[0][p][i] = a0.mul() + a1.mul();
+                if (p == 0) S.c0[i] = B[0];
+            }
             gbar<G>(g);
-            // (d) diagonal block A(R_s, R_s) <- H^H A H
-            sbr_two_sided<R, C, BMAX, G, P>(S, vc, tau, l, Hg, ldi, r, tid, g, s == 0 ? dd + j + 1 : nullptr);
+            // (b) the reflector.  With C1 = B H(j,s-1) = B - tau_p y v_p^H, x = C1(:, 0) gives H(j,s);
+            // then H^H C1 = B - tau_p y v_p^H - conj(tau) v r with r_k = (v^H B)_k - gamma conj(v_p,k),
+            // gamma = v^H (tau_p y).  At s = 0 x is column j below the diagonal.
+            C vl[SL], ty[SL];
+            R beta = R(0);
+            if (warp == 0) {
+                R part = R(0);
+                if (s > 0) {
+#pragma unroll
+                    for (int u = 0; u < SL; ++u) {
+                        const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                        C y = S.red[0][0][e];
+#pragma unroll
+                        for (int q = 1; q < P; ++q) y = y + S.red[0][q][e];
+                        ty[u] = taup * y;
+                        x[u] = S.c0[e] - ty[u];   // v_p[0] = 1
+                        S.ty[e] = ty[u];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < SL; ++u)
+                    if (u > 0 || (BMAX >= 32 ? lane : lane % BMAX) > 0) part += abs2(x[u]);
+                const R xn2 = lane_sum<BMAX>(part);
+                const C alpha = mk(__shfl_sync(0xffffffffu, x[0].x, 0), __shfl_sync(0xffffffffu, x[0].y, 0));
+                C scale;
+                make_reflector<R, C>(alpha, xn2, tau, beta, scale);
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    vl[u] = e == 0 ? mk(R(1), R(0)) : x[u] * scale;
+                    S.v[cur][e] = DupC::of(vl[u]);
+                }
+                if (lane == 0) S.beta[0] = mk(beta, R(0));
+            }
+            gbar<G>(g);
+            const auto* v = S.v[cur];
+            // (c) column i over rows k0 .. k0 + EL - 1 of B and of D's strict lower triangle, and row i
+            // of D's lower triangle over columns k0 .. (warps whose share is zero skip it)
+            {
+                SbrAcc<C> zu0, zu1, zc0, zc1, zr0, zr1;
+#pragma unroll
+                for (int q = 0; q < EL; q += 2) {
+                    if (F64 && k0 + q >= l) continue;
+                    const auto v0 = v[k0 + q], v1 = v[k0 + q + 1];
+                    C b0, b1;
+                    if (s > 0) {
+                        ld_pair(&S.B[i * LD + k0 + q], b0, b1);
+                        zu0.addc(b0, v0);
+                        zu1.addc(b1, v1);
+                    }
+                    if (low) {
+                        ld_pair(&S.D[i * LD + k0 + q], b0, b1);
+                        zc0.addc(b0, v0);
+                        zc1.addc(b1, v1);
+                    }
+                    if (row) {
+                        zr0.add(D[q], v0);
+                        zr1.add(D[q + 1], v1);
+                    }
+                }
+                if (s > 0) S.red[1][p][i] = zu0.mulc() + zu1.mulc();
+                S.red[2][p][i] = (zr0.mul() + zr1.mul()) + conj(zc0.mulc() + zc1.mulc());
+            }
+            C gam = zero;
+            if (warp == 0 && s > 0) {  // gamma, while the other warps are at their sums
+                R gre = R(0), gim = R(0);
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const C gc = cmulc(vl[u], ty[u]);
+                    gre += gc.x;
+                    gim += gc.y;
+                }
+                gam = mk(lane_sum<BMAX>(gre), lane_sum<BMAX>(gim));
+            }
+            gbar<G>(g);
+            // (d) w_u = conj(tau) r for B; D <- H^H D H = D - v w^H - w v^H with y = D v,
+            // w = tau y - |tau|^2 (v^H y) / 2 v
+            if (warp == 0) {
+                C y2[SL];
+                R part = R(0);
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    y2[u] = S.red[2][0][e];
+#pragma unroll
+                    for (int q = 1; q < P; ++q) y2[u] = y2[u] + S.red[2][q][e];
+                    part += vl[u].x * y2[u].x + vl[u].y * y2[u].y;  // Re(conj(v) y)
+                    if (s > 0) {
+                        C z = S.red[1][0][e];
+#pragma unroll
+                        for (int q = 1; q < P; ++q) z = z + S.red[1][q][e];
+                        S.wu[e] = DupC::of(conj(tau) * (z - gam * conj(DupC::val(S.v[cur ^ 1][e]))));
+                    }
+                }
+                const R t2 = R(0.5) * abs2(tau) * lane_sum<BMAX>(part);
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    S.wd[e] = DupC::of(tau * y2[u] - t2 * vl[u]);
+                }
+            }
+            gbar<G>(g);
+            // (e) rank-2 updates of this thread's entries, back to global memory
+            const C vi = DupC::val(v[i]), wi = DupC::val(S.wd[i]);
+            if (s > 0) {
+                const C tyi = S.ty[i];
+                const auto *vp = S.v[cur ^ 1] + k0, *wu = S.wu + k0;
+                C* h = Hg + (rp + k0) * ldi + r + i;
+#pragma unroll
+                for (int q = 0; q < EL; ++q) {
+                    if (F64 && k0 + q >= b) continue;
+                    C a = sbr_sub(sbr_sub_conj(B[q], tyi, vp[q]), vi, wu[q]);
+                    if (q == 0 && p == 0) a = i == 0 ? S.beta[0] : zero;
+                    st_if(h + q * ldi, a, i < l && k0 + q < b);
+                }
+            }
+            if (row) {
+                const auto *vk = v + k0, *wd = S.wd + k0;
+                C* h = Hg + (r + k0) * ldi + r + i;
+#pragma unroll
+                for (int q = 0; q < EL; ++q) {
+                    const int k = k0 + q;
+                    if (F64 && k >= l) continue;
+                    // v_i conj(w_k) + w_i conj(v_k)
+                    C a = sbr_sub_conj(sbr_sub_conj(D[q], vi, wd[q]), wi, vk[q]);
+                    if (i == k) a.y = R(0);
+                    st_if(h + q * ldi, a, i >= k && i < l);
+                    if (q == 0 && s == 0 && tid == 0) dd[j + 1] = (double)a.x;
+                }
+            }
+            if (warp == 0) {
+                if (s == 0) {
+#pragma unroll
+                    for (int u = 0; u < SL; ++u) {
+                        const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                        if (e < l) Hg[j * ldi + r + e] = e == 0 ? mk(beta, R(0)) : zero;
+                    }
+                    if (lane == 0) ee[j] = (double)beta;
+                }
+                // store the reflector for the back-transform, marked evict-first: the store is
+                // written once and read only after the chase, and L2 should keep the band's lines
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    if (e < b) __stcs(&V[(sbr_off(n, b, s) + j) * b + e], vl[u]);
+                }
+                if (lane == 0) __stcs(&T[sbr_off(n, b, s) + j], tau);
+            }
+            taup = tau;
             cur ^= 1;
-            if (CL > 1) __threadfence(); else __threadfence_block();  // the step's writes, then its key
-            gbar<G>(g);
-            if (tid == 0) key[g] = (long long)j * KK + (s + 1 == nsteps ? KK - 1 : s + 1);
+            gbar<G>(g);  // the group's writes, then (release) its key
+            if (tid == G - 1) key_store(mykey, (long long)j * KK + (s + 1 == nsteps ? KK - 1 : s + 1));
         }
     }
-    // the partner may still read this CTA's keys and abort flag: leave together
+    // other CTAs may still read this CTA's keys and abort flag: leave together
     if (CL > 1) cluster.sync();
 }
 
@@ -616,18 +703,20 @@ __global__ void __launch_bounds__(256) k_sbr_out(const MmfDesc* __restrict__ des
 }
 
 // ------------------------------------------------------------------ launchers
-template <class R, int BMAX, int G, int NG, int CL>
-static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
-                                int* status) {
+// The chase with CL CTAs per system; *fits (if given) only reports whether count clusters of that
+// size are resident at once (a second wave would double the time).
+template <class R, int BMAX, int P, int NG, int CL>
+static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
+                                   int* status, bool* fits) {
     typedef typename Cx<R>::T C;
-    static_assert(sizeof(SbrGroup<C, BMAX, G / BMAX>) % 16 == 0, "group blocks keep 16-byte alignment");
-    const size_t sm = sbr_hdr(NG) + sizeof(SbrGroup<C, BMAX, G / BMAX>) * NG;
-    cudaError_t e = cudaFuncSetAttribute(k_sbr_chase<R, BMAX, G, NG, CL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    static_assert(sizeof(SbrGroup<C, BMAX, P>) % 16 == 0, "group blocks keep 16-byte alignment");
+    const size_t sm = sbr_hdr(NG) + sizeof(SbrGroup<C, BMAX, P>) * NG;
+    auto kern = k_sbr_chase<R, BMAX, P, NG, CL>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(L.count * CL);
-    cfg.blockDim = dim3(G * NG);
+    cfg.blockDim = dim3(BMAX * P * NG);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
@@ -637,8 +726,41 @@ static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, dou
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_sbr_chase<R, BMAX, G, NG, CL>, L.desc, L.idx, (C*)H, (C*)store, dvec, evec,
-                              status);
+    if (fits) {
+        int nc = 0;
+        e = cudaOccupancyMaxActiveClusters(&nc, kern, &cfg);
+        *fits = e == cudaSuccess && L.count <= nc;
+        return e;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, L.desc, L.idx, (C*)H, (C*)store, dvec, evec, status);
+}
+
+// The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
+// pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
+// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
+// take, with 8 it takes 15.5; in FP64 eight systems take 455 ms on 2 CTAs each, 147 on 8.
+template <class R, int BMAX, int P, int NG>
+static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
+                                int* status) {
+    const int sweeps = L.nmax / BMAX + 1;  // b > BMAX / 2, so at least n / (2 b)
+    bool fits = false;
+    cudaError_t e = cudaSuccess;
+    if (sweeps > 4 * NG) {
+        e = launch_chase_cl<R, BMAX, P, NG, 8>(L, H, store, dvec, evec, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_chase_cl<R, BMAX, P, NG, 8>(L, H, store, dvec, evec, status, nullptr);
+    }
+    if (sweeps > 2 * NG) {
+        e = launch_chase_cl<R, BMAX, P, NG, 4>(L, H, store, dvec, evec, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_chase_cl<R, BMAX, P, NG, 4>(L, H, store, dvec, evec, status, nullptr);
+    }
+    if (sweeps > NG) {
+        e = launch_chase_cl<R, BMAX, P, NG, 2>(L, H, store, dvec, evec, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_chase_cl<R, BMAX, P, NG, 2>(L, H, store, dvec, evec, status, nullptr);
+    }
+    return launch_chase_cl<R, BMAX, P, NG, 1>(L, H, store, dvec, evec, status, nullptr);
 }
 
 template <int BMAX>
@@ -655,44 +777,24 @@ static cudaError_t launch_bt(const MmfLaunch& L, const double2* store, const dou
     return cudaGetLastError();
 }
 
-// The paired (two-SM) chase can be switched off for comparison: MMF_SBR_PAIRS=0 in the
-// environment.
-static bool sbr_pairs_enabled() {
-    static int v = -1;
-    if (v < 0) {
-        const char* e = getenv("MMF_SBR_PAIRS");
-        v = (e && e[0] == '0') ? 0 : 1;
-    }
-    return v == 1;
-}
-
 int mmf_sbr_class(int b) { return b <= 8 ? 8 : b <= 16 ? 16 : b <= 32 ? 32 : b <= 64 ? 64 : 0; }
 
 cudaError_t mmf_launch_sbr_chase(const MmfLaunch& L, int bmax, void* H, double2* store, double* dvec, double* evec,
                                  int* status, int fp32) {
     if (L.count <= 0) return cudaSuccess;
-    // two CTAs (SMs) per system for the widest band while the pairs fit the GPU in one wave
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const bool pair = sbr_pairs_enabled() && 2 * L.count <= sms;
     if (fp32) {
         switch (bmax) {
-            case 8: return launch_chase<float, 8, 32, 15, 1>(L, H, store, dvec, evec, status);
-            case 16: return launch_chase<float, 16, 32, 15, 1>(L, H, store, dvec, evec, status);
-            case 32: return launch_chase<float, 32, 64, 8, 1>(L, H, store, dvec, evec, status);
-            case 64:
-                return pair ? launch_chase<float, 64, 128, 3, 2>(L, H, store, dvec, evec, status)
-                            : launch_chase<float, 64, 128, 3, 1>(L, H, store, dvec, evec, status);
+            case 8: return launch_chase<float, 8, 4, 16>(L, H, store, dvec, evec, status);
+            case 16: return launch_chase<float, 16, 2, 16>(L, H, store, dvec, evec, status);
+            case 32: return launch_chase<float, 32, 4, 4>(L, H, store, dvec, evec, status);
+            case 64: return launch_chase<float, 64, 4, 2>(L, H, store, dvec, evec, status);
         }
     } else {
         switch (bmax) {
-            case 8: return launch_chase<double, 8, 32, 15, 1>(L, H, store, dvec, evec, status);
-            case 16: return launch_chase<double, 16, 32, 12, 1>(L, H, store, dvec, evec, status);
-            case 32: return launch_chase<double, 32, 64, 4, 1>(L, H, store, dvec, evec, status);
-            case 64:
-                return pair ? launch_chase<double, 64, 128, 1, 2>(L, H, store, dvec, evec, status)
-                            : launch_chase<double, 64, 128, 1, 1>(L, H, store, dvec, evec, status);
+            case 8: return launch_chase<double, 8, 4, 16>(L, H, store, dvec, evec, status);
+            case 16: return launch_chase<double, 16, 2, 8>(L, H, store, dvec, evec, status);
+            case 32: return launch_chase<double, 32, 4, 4>(L, H, store, dvec, evec, status);
+            case 64: return launch_chase<double, 64, 4, 1>(L, H, store, dvec, evec, status);
         }
     }
     return cudaErrorInvalidValue;
