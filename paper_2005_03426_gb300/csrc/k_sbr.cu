@@ -199,28 +199,6 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
     b = p[1];
 }
 
-template <class R> __device__ __forceinline__ R rsqrt_of(R x);
-template <> __device__ __forceinline__ float rsqrt_of<float>(float x) { return sqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_of<double>(double x) { return sqrt(x); }
-
-// Householder of x = (alpha, rest) with ||rest||^2 = xn2: H^H x = beta e1, beta real.
-// Returns tau and beta; scale = 1 / (alpha - beta) multiplies rest into v.
-template <class R, class C>
-__device__ __forceinline__ void make_reflector(C alpha, R xn2, C& tau, R& beta, C& scale) {
-    if (xn2 == R(0) && alpha.y == R(0)) {
-        tau = mk(R(0), R(0));
-        beta = alpha.x;
-        scale = mk(R(0), R(0));
-        return;
-    }
-    const R nrm = rsqrt_of<R>(alpha.x * alpha.x + alpha.y * alpha.y + xn2);
-    beta = alpha.x >= R(0) ? -nrm : nrm;
-    tau = mk((beta - alpha.x) / beta, -alpha.y / beta);
-    const C den = mk(alpha.x - beta, alpha.y);
-    const R dd = den.x * den.x + den.y * den.y;
-    scale = mk(den.x / dd, -den.y / dd);
-}
-
 // One group of G = BMAX P threads per sweep: thread (i, p) keeps row i, columns p EL .. p EL + EL - 1
 // of the step's two blocks B = A(R_s, R_{s-1}) and D = A(R_s, R_s) (lower triangle) in registers,
 // from its loads to its stores; a copy in shared memory serves the sums down the columns.  A step is
@@ -384,7 +362,7 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                 const R xn2 = lane_sum<BMAX>(part);
                 const C alpha = mk(__shfl_sync(0xffffffffu, x[0].x, 0), __shfl_sync(0xffffffffu, x[0].y, 0));
                 C scale;
-                make_reflector<R, C>(alpha, xn2, tau, beta, scale);
+                warp_reflector<R, C>(alpha, xn2, lane, tau, beta, scale);
 #pragma unroll
                 for (int u = 0; u < SL; ++u) {
                     const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
@@ -738,7 +716,7 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
 // The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
 // pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
 // system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
-// take, with 8 it takes 15.5; in FP64 eight systems take 455 ms on 2 CTAs each, 147 on 8.
+// take, with 8 it takes 15.5.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
                                 int* status) {

@@ -90,7 +90,7 @@ struct mmf_batch {
     int count = 0, precision = 0, nt = 0;
     std::vector<mmf_sys*> sys;
     std::vector<MmfDesc> desc;
-    std::vector<int> all, small, large, medium, huge;  // large = medium + huge + the banded ones
+    std::vector<int> all, small, large, medium, tiny, huge;  // large = medium + tiny + huge + the banded ones
     // banded systems reduced by the bulge chase, per window class (8, 16, 32, 64)
     std::vector<int> sbr[4];
     int nmax_sbr[4] = {0, 0, 0, 0};
@@ -119,9 +119,10 @@ struct mmf_batch {
     unsigned char* base = nullptr;
     size_t bytes = 0;
     MmfDesc* d_desc = nullptr;
-    int *d_all = nullptr, *d_small = nullptr, *d_large = nullptr, *d_medium = nullptr, *d_status = nullptr;
+    int *d_all = nullptr, *d_small = nullptr, *d_large = nullptr, *d_medium = nullptr, *d_tiny = nullptr,
+        *d_status = nullptr;
     int *d_rband = nullptr, *d_rfull = nullptr;
-    int nmax_medium = 0;
+    int nmax_medium = 0, nmax_tiny = 0;
     double2* d_coef = nullptr;
     void* d_H = nullptr;
     double2* d_Zf = nullptr;
@@ -654,11 +655,16 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
         b->n_p += (int64_t)s->D * s->D;
         b->all.push_back(i);
         (d.small ? b->small : b->large).push_back(i);
-        if (!d.small && !cls) (n >= lmin ? b->huge : b->medium).push_back(i);
+        // dense reduction: whole GPU, one CTA with the matrix in shared memory, or a cluster
+        const bool one_cta = n <= mmf_hetrd_small_n(fp32);
+        if (!d.small && !cls) (n >= lmin ? b->huge : one_cta ? b->tiny : b->medium).push_back(i);
         b->nmax_all = std::max(b->nmax_all, (int)n);
         if (d.small) b->nmax_small = std::max(b->nmax_small, (int)n);
         else b->nmax_large = std::max(b->nmax_large, (int)n);
-        if (!d.small && !cls && n < lmin) b->nmax_medium = std::max(b->nmax_medium, (int)n);
+        if (!d.small && !cls && n < lmin) {
+            int& nm = one_cta ? b->nmax_tiny : b->nmax_medium;
+            nm = std::max(nm, (int)n);
+        }
         b->Mmax = std::max(b->Mmax, (int)M);
         b->Dmax = std::max(b->Dmax, s->D);
         if (n >= refine_full_n(ctx)) {
@@ -674,7 +680,7 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
     Pool p;
     size_t o_desc = p.take(sizeof(MmfDesc) * count);
     size_t o_all = p.take(sizeof(int) * count), o_small = p.take(sizeof(int) * count),
-           o_large = p.take(sizeof(int) * count), o_medium = p.take(sizeof(int) * count),
+           o_large = p.take(sizeof(int) * count), o_medium = p.take(sizeof(int) * count), o_tiny = p.take(sizeof(int) * count),
            o_status = p.take(sizeof(int) * count), o_rband = p.take(sizeof(int) * count),
            o_rfull = p.take(sizeof(int) * count), o_sbr = p.take(sizeof(int) * count), o_sbt = p.take(sizeof(int) * count),
            o_btc = p.take(sizeof(int) * count),
@@ -744,6 +750,7 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
     b->d_small = (int*)(B + o_small);
     b->d_large = (int*)(B + o_large);
     b->d_medium = (int*)(B + o_medium);
+    b->d_tiny = (int*)(B + o_tiny);
     b->d_status = (int*)(B + o_status);
     b->d_rband = (int*)(B + o_rband);
     b->d_rfull = (int*)(B + o_rfull);
@@ -821,6 +828,8 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
         e = cudaMemcpyAsync(b->d_large, b->large.data(), sizeof(int) * b->large.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !b->medium.empty())
         e = cudaMemcpyAsync(b->d_medium, b->medium.data(), sizeof(int) * b->medium.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !b->tiny.empty())
+        e = cudaMemcpyAsync(b->d_tiny, b->tiny.data(), sizeof(int) * b->tiny.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !b->rband.empty())
         e = cudaMemcpyAsync(b->d_rband, b->rband.data(), sizeof(int) * b->rband.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !b->rfull.empty())
@@ -990,6 +999,10 @@ static int stage_eig(mmf_batch* b) {
             LAUNCH(mmf_launch_hetrd(Lm, b->d_H, b->d_Vp, b->d_Wp, b->d_d, b->d_e, b->d_tau, fp32, b->hetrd_tc,
                                     b->d_status),
                    1);
+        }
+        if (!b->tiny.empty()) {
+            MmfLaunch Lt = launch_of(b, b->tiny, b->d_tiny, b->nmax_tiny);
+            LAUNCH(mmf_launch_hetrd_small(Lt, b->d_H, b->d_d, b->d_e, b->d_tau, fp32), 1);
         }
         for (int ci = 0; ci < 4; ++ci) {  // banded systems: bulge chase
             if (b->sbr[ci].empty()) continue;

@@ -87,6 +87,30 @@ template <class R> __device__ __forceinline__ R warp_sum(R v) {
     return v;
 }
 
+// Householder of x = (alpha, rest) with ||rest||^2 = xn2, for a whole warp (same arguments in every
+// lane): H^H x = beta e1 with beta real, H = I - tau v v^H, v = (1, rest scale),
+//   beta = -sign(Re alpha) sqrt(|alpha|^2 + xn2), tau = (beta - alpha) / beta, scale = 1 / (alpha - beta).
+// The four divisions run in four lanes at once (a division costs 650 cycles in FP64).
+__device__ __forceinline__ float sqrt_of(float x) { return sqrtf(x); }
+__device__ __forceinline__ double sqrt_of(double x) { return sqrt(x); }
+template <class R, class C>
+__device__ __forceinline__ void warp_reflector(C alpha, R xn2, int lane, C& tau, R& beta, C& scale) {
+    if (xn2 == R(0) && alpha.y == R(0)) {
+        tau = mk(R(0), R(0));
+        beta = alpha.x;
+        scale = mk(R(0), R(0));
+        return;
+    }
+    const R nrm = sqrt_of(alpha.x * alpha.x + alpha.y * alpha.y + xn2);
+    beta = alpha.x >= R(0) ? -nrm : nrm;
+    const R dx = alpha.x - beta, dd = dx * dx + alpha.y * alpha.y;
+    const int q = lane & 3;
+    const R num = q == 0 ? beta - alpha.x : q == 2 ? dx : -alpha.y;
+    const R r = num / (q < 2 ? beta : dd);
+    tau = mk(__shfl_sync(0xffffffffu, r, 0), __shfl_sync(0xffffffffu, r, 1));
+    scale = mk(__shfl_sync(0xffffffffu, r, 2), __shfl_sync(0xffffffffu, r, 3));
+}
+
 // Fourier vector of block b: n_k = (b / S_k) mod (2N_k+1) - N_k
 __device__ __forceinline__ void block_nvec(const MmfDesc& d, int b, int* nv) {
 #pragma unroll
@@ -240,6 +264,10 @@ cudaError_t mmf_launch_outputs(const MmfLaunch& L, int Mmax, int Dmax, const dou
                                double2* F, double2* U, double* P, double cluster_rel, int skip_u,
                                void* scratch, int scratch_esz);
 int mmf_hetrd_max_n(int fp32);
+// the same reduction with the whole matrix in one CTA's shared memory (k_hetrd_small.cu), for n up to
+// mmf_hetrd_small_n
+int mmf_hetrd_small_n(int fp32);
+cudaError_t mmf_launch_hetrd_small(const MmfLaunch& L, void* H, double* dvec, double* evec, void* tau, int fp32);
 // banded H_F (k_sbr.cu): bulge chase to real tridiagonal form (d, e; reflectors kept in the
 // system's FP64 eigenvector slot), then Z = Q Y into the back-transform's output (Zp)
 int mmf_sbr_class(int band);                 // window class 8/16/32/64, 0 if the band is wider
