@@ -17,13 +17,19 @@
 // Result: d (diagonal), e = beta (sub-diagonal, real), tau, and v[k+2:] stored in
 // A(k+2:, k).  Q = P_0 P_1 ... P_{n-2}, Q^H H_F Q = tridiag(e, d, e).
 //
-// One thread-block cluster of CL CTAs (512 threads each) per system.  The hemv streams the
-// lower triangle of the trailing matrix once per column with coalesced column reads: a warp
-// owns 8 columns, lanes own rows, the row part accumulates through shared-memory atomics and
-// the column part by warp-shuffle reductions.  With CL = 2 the two CTAs of the cluster split the
-// column blocks of the hemv, the rows of the column update and the tiles of the trailing
-// update; each adds its partner's partial hemv result through distributed shared memory and
-// repeats the short O(m) vector steps itself.
+// One thread-block cluster of CL CTAs (512 threads each, CL = 1, 2, 4 or 8) per system.  The hemv
+// streams the lower triangle of the trailing matrix once per column with coalesced column reads: a
+// warp owns 8 columns, lanes own rows, the row part accumulates through shared-memory atomics and
+// the column part by warp-shuffle reductions.  The CTAs split the column blocks of the hemv and the
+// tiles of the trailing update; everything of length m is split by rows (chunks of 32 rows dealt
+// round-robin): the pending panel updates of the column, the dot products W^H v and V^H v, and the
+// corrections of y.  Per column three cluster barriers: the column and its norm reach every CTA
+// (pushed through distributed shared memory); the partial hemv results and dot products are
+// complete; the scalar w^H v is complete.
+//
+// What bounds it: with one system per two SMs the hemv's L2 reads and the 2i column reads of the
+// panel, repeated by each CTA; with 8 SMs a system the barriers and L2 latencies of a column (a few
+// microseconds), which is why the split reaches the O(m i) steps too.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -37,8 +43,8 @@ namespace cg = cooperative_groups;
 
 #define HT_THREADS 512
 #define HT_TILE 64
-#define HT_SEG 512   // rows per hemv task (a multiple of 64)
-
+#define HT_CL4_N 256   // smallest n reduced by 4 / 8 CTAs per system
+#define HT_CL8_N 384
 template <class R>
 __device__ __forceinline__ R block_sum(R v, R* red) {
     v = warp_sum(v);
@@ -56,10 +62,6 @@ __device__ __forceinline__ R block_sum(R v, R* red) {
 }
 
 
-// FP32 hemv pipeline: per warp two stages of HT_CH rows x 8 columns, filled by cp.async
-#define HT_CH 64
-#define HT_STAGE_ELEMS (8 * HT_CH)
-
 template <class R>
 __host__ __device__ constexpr size_t ht_fixed_bytes() {
     return sizeof(typename Cx<R>::T) * (4 * MMF_NB + 4) + sizeof(R) * 72;
@@ -69,21 +71,15 @@ __host__ __device__ inline size_t ht_big_offset(int nmax) {
     const size_t o = sizeof(typename Cx<R>::T) * 3 * (size_t)nmax + ht_fixed_bytes<R>();
     return (o + 15) & ~(size_t)15;
 }
-// FP32: the hemv's cp.async stages, or (tensor-core trailing update) two operand stages of 64 KB
-// at a 1024-byte boundary
+// the partial sums of the O(m i) steps, or the trailing update's operands: FP32 two stages of 64 KB
+// at a 1024-byte boundary (tensor cores), FP64 four 32 x 64 tiles
 #define HT_TC_STAGE 65536u
 template <class R>
 __host__ __device__ constexpr size_t ht_big_bytes() {
-    return sizeof(R) == 4 ? (size_t)(HT_THREADS / 32) * 2 * HT_STAGE_ELEMS * sizeof(typename Cx<R>::T) + 1024
+    return sizeof(R) == 4 ? (size_t)2 * HT_TC_STAGE + 1024
                           : (size_t)4 * MMF_NB * HT_TILE * sizeof(typename Cx<R>::T);
 }
-static_assert((HT_THREADS / 32) * 2 * HT_STAGE_ELEMS * 8 >= 2 * HT_TC_STAGE, "tensor-core stages fit");
-
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc, int src_bytes) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(gsrc), "r"(src_bytes) : "memory");
-}
-static_assert(4 * MMF_NB * HT_TILE <= (HT_THREADS / 32) * 2 * HT_STAGE_ELEMS, "her2k tiles fit the hemv stages");
+static_assert(4 * MMF_NB * HT_TILE * sizeof(float2) <= 2 * HT_TC_STAGE, "FP32-unit tiles fit");
 
 // two block-wide sums in one pass (red holds 2 x 33 values)
 template <class R>
@@ -121,152 +117,131 @@ __device__ __forceinline__ void atomic_add_c(float2* p, float2 v) {
 }
 
 
-// FP32 hemv share of one warp, pipelined through shared memory: the warp's chunks (HT_CH rows x
-// 8 columns of its row-segment tasks) are copied by cp.async one chunk ahead of the arithmetic,
-// so the trailing matrix streams while the previous chunk is multiplied.  Task h of the CTA:
-// column block (rank + CL (h % nloc)) of 8 columns, rows from segment h / nloc (HT_SEG rows).
-// The arithmetic is branch-free outside the diagonal chunk: the block's 8 entries of v are held
-// in registers per task, the chunk's operands are read from shared memory before the FMAs.
-// Complex products use packed FP32 pair FMAs with split accumulators: for a row r,
-// y_r += sum_jj a v_jj is kept as r1 = sum a (v.x, v.x), r2 = sum a (v.y, v.y), y_r += (r1.x - r2.y,
-// r1.y + r2.x); for a column, sum_r conj(a) v_r as c1 = sum a (v_r.x, v_r.x), c2 = sum a (v_r.y,
-// v_r.y), added as (c1.x + c2.y, c2.x - c1.y).
-struct HtTask {
-    int c0, rbeg, rend, nc;
+// One warp's share of y = A22 v: tasks of 32 RPL rows (RPL rows per lane: 4 in FP32, 2 in FP64) x cw
+// columns on and below the diagonal, dealt round-robin over the warps of all CTAs.  A task goes by in
+// blocks of 8 columns, HT_NL columns loading (L2) at a time.  The row part stays in registers over
+// the task; the column parts of a block are summed over the lanes by one butterfly that halves the
+// values at each exchange.  A warp's time is the latency of its chain
+// of loads and exchanges (L2 latency near 1000 cycles), so few long steps beat many short ones: at
+// m = 1000 on 8 SMs 9 us, 27 bytes a clock and SM, where blocks of 4 columns with an exchange and two
+// in flight take 12; a ring of cp.async pieces 7 columns deep takes 15 (its instructions per column).
+// (HT_NL = 8 measures the same and needs more registers.)  cw is chosen so that every warp gets a few
+// tasks.
+// FP32: complex products as packed pair FMAs with split accumulators p = sum (a.x v.x, a.y v.y) and
+// q = sum (a.x v.y, a.y v.x): sum a v = (p.x - p.y, q.x + q.y), sum conj(a) v = (p.x + p.y, q.x - q.y).
+#define HT_NL 4
+template <class C> struct HtAcc;  // running sum of products of entries with entries of v
+template <> struct HtAcc<float2> {
+    float2 p, q;
+    __device__ __forceinline__ HtAcc() : p(make_float2(0.f, 0.f)), q(make_float2(0.f, 0.f)) {}
+    __device__ __forceinline__ void add(float2 a, float2 v, float2 vs) {  // vs = (v.y, v.x)
+        p = __ffma2_rn(a, v, p);
+        q = __ffma2_rn(a, vs, q);
+    }
+    __device__ __forceinline__ void addc(float2 a, float2 v, float2 vs) { add(a, v, vs); }
+    __device__ __forceinline__ float2 mul() const { return make_float2(p.x - p.y, q.x + q.y); }   // sum a v
+    __device__ __forceinline__ float2 mulc() const { return make_float2(p.x + p.y, q.x - q.y); }  // sum conj(a) v
+};
+template <> struct HtAcc<double2> {
+    double2 p;
+    __device__ __forceinline__ HtAcc() : p(make_double2(0.0, 0.0)) {}
+    __device__ __forceinline__ void add(double2 a, double2 v, double2) { p = p + a * v; }
+    __device__ __forceinline__ void addc(double2 a, double2 v, double2) { p = p + cmulc(a, v); }
+    __device__ __forceinline__ double2 mul() const { return p; }
+    __device__ __forceinline__ double2 mulc() const { return p; }
 };
 
-__device__ __forceinline__ bool ht_task(int h, int nloc, int rank, int CL, int m, HtTask& t) {
-    const int qb = h % nloc, sg = h / nloc;
-    t.c0 = (rank + CL * qb) << 3;
-    t.rbeg = t.c0 + sg * HT_SEG;
-    t.rend = min(t.rbeg + HT_SEG, m);
-    t.nc = min(8, m - t.c0);
-    return t.rbeg < m;
+// a lane's entries of columns c .. c + NL - 1, rows r + 32 h; a task on the diagonal takes the lower
+// triangle and the (real) diagonal only
+template <class C, int RPL, int NL, bool DIAG>
+__device__ __forceinline__ void ht_load(const C* __restrict__ p, int ld, int m, int r, int c, C (&a)[NL * RPL]) {
+#pragma unroll
+    for (int j = 0; j < NL; ++j)
+#pragma unroll
+        for (int h = 0; h < RPL; ++h) {
+            C x = czero<C>();
+            if (r + 32 * h < m && (!DIAG || r + 32 * h >= c + j)) x = __ldcg(p + (int64_t)j * ld + 32 * h);
+            if (DIAG && r + 32 * h == c + j) x.y = 0;
+            a[j * RPL + h] = x;
+        }
 }
 
-__device__ __forceinline__ void ht_issue(const float2* __restrict__ a22, int ld, const HtTask& t, int r0,
-                                         float2* buf, int lane) {
-    const float2* colbase = a22 + (int64_t)t.c0 * ld;
-    if (r0 >= t.c0 + 8 && r0 + HT_CH <= t.rend && t.nc == 8) {
-        // the common chunk: below the diagonal block, inside the task, all 8 columns present
-        const float2* p = colbase + r0 + lane;
+template <class R, class C, int RPL, bool DIAG>
+__device__ __forceinline__ void ht_task(const C* __restrict__ a22, int ld, int m, const C* __restrict__ vS, C* yS,
+                                        int r, int c0, int cw, int lane) {
+    constexpr int NL = HT_NL;
+    C v[RPL], vs[RPL], a[NL * RPL];
+    HtAcc<C> y[RPL];
+    const C* p = a22 + (int64_t)c0 * ld + r;
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj)
-#pragma unroll
-            for (int hf = 0; hf < HT_CH / 32; ++hf)
-                cp_async8(buf + jj * HT_CH + lane + 32 * hf, p + (int64_t)jj * ld + 32 * hf, 8);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        return;
+    for (int h = 0; h < RPL; ++h) {
+        v[h] = r + 32 * h < m ? vS[r + 32 * h] : czero<C>();
+        vs[h] = mk(v[h].y, v[h].x);
     }
+#pragma unroll 1
+    for (int cb = c0; cb < c0 + cw; cb += 8) {
+        R z[16];
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
+        for (int b = 0; b < 8; b += NL) {
+            ht_load<C, RPL, NL, DIAG>(p, ld, m, r, cb + b, a);
+            p += NL * (int64_t)ld;
 #pragma unroll
-        for (int hf = 0; hf < HT_CH / 32; ++hf) {
-            const int row = r0 + lane + 32 * hf;
-            const bool ok = jj < t.nc && row < t.rend && row >= t.c0 + jj;
-            const float2* src = ok ? colbase + (int64_t)jj * ld + row : a22;
-            cp_async8(buf + jj * HT_CH + lane + 32 * hf, src, ok ? 8 : 0);
+            for (int j = 0; j < NL; ++j) {
+                const int c = cb + b + j;
+                const C vc = vS[DIAG ? min(c, m - 1) : c];
+                const C vcs = mk(vc.y, vc.x);
+                HtAcc<C> s;
+#pragma unroll
+                for (int h = 0; h < RPL; ++h) {
+                    y[h].add(a[j * RPL + h], vc, vcs);
+                    // the diagonal entry counts once, in the row part
+                    s.addc(DIAG && r + 32 * h == c ? czero<C>() : a[j * RPL + h], v[h], vs[h]);
+                }
+                const C f = s.mulc();
+                z[2 * (b + j)] = f.x;
+                z[2 * (b + j) + 1] = f.y;
+            }
         }
+        // lanes with bit o of their number set keep the upper half of the values
+#pragma unroll
+        for (int o = 16; o >= 2; o >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int e = 0; e < o / 2; ++e) {
+                const R keep = up ? z[e + o / 2] : z[e], send = up ? z[e] : z[e + o / 2];
+                z[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+        z[0] += __shfl_xor_sync(0xffffffffu, z[0], 1);
+        // lanes 2 q and 2 q + 1 hold value q: re / im (bit 0) of column cb + q / 2
+        const int c = cb + (lane >> 2);
+        if (!(lane & 1) && (!DIAG || c < m)) atomicAdd(reinterpret_cast<R*>(&yS[c]) + ((lane >> 1) & 1), z[0]);
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+    for (int h = 0; h < RPL; ++h)
+        if (r + 32 * h < m) atomic_add_c(&yS[r + 32 * h], y[h].mul());
 }
 
-__device__ int hemv_f32_staged(const float2* __restrict__ a22, int ld, int m, const float2* __restrict__ vS,
-                               float2* yS, float2* stg, int rank, int CL, int nloc, int nseg, int warp, int lane) {
-    const int NW = HT_THREADS / 32;
-    const int nh = nloc * nseg;
-    // the warp's first valid task
-    int h = warp;
-    HtTask t;
-    while (h < nh && !ht_task(h, nloc, rank, CL, m, t)) h += NW;
-    if (h >= nh) return 0;
-    int r0 = t.rbeg, buf = 0, nchunks = 0;
-    ht_issue(a22, ld, t, r0, stg, lane);
-    float2 v[8], vxx[8], vyy[8], c1[8], c2[8];
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-        v[jj] = (jj < t.nc) ? vS[t.c0 + jj] : czero<float2>();
-        vxx[jj] = make_float2(v[jj].x, v[jj].x);
-        vyy[jj] = make_float2(v[jj].y, v[jj].y);
-        c1[jj] = c2[jj] = czero<float2>();
+template <class R, class C>
+__device__ __forceinline__ void ht_hemv(const C* __restrict__ a22, int ld, int m, const C* __restrict__ vS, C* yS,
+                                        int wid, int nw, int lane) {
+    constexpr int RPL = sizeof(R) == 4 ? 4 : 2, TR = 32 * RPL;
+    // columns per task: about three tasks for each warp, within 16 .. 64
+    const int want = (int)((int64_t)m * m / (2 * TR * 3) / nw);
+    const int cw = want < 24 ? 16 : want < 48 ? 32 : 64, G = TR / cw;
+    const int nt = (m + TR - 1) / TR;
+    const int ntask = nt * (nt + 1) / 2 * G;
+    for (int t = wid; t < ntask; t += nw) {
+        const int tt = t / G;
+        int ti = (int)((sqrtf(8.0f * (float)tt + 1.0f) - 1.0f) * 0.5f);
+        while ((ti + 1) * (ti + 2) / 2 <= tt) ++ti;
+        while (ti * (ti + 1) / 2 > tt) --ti;
+        const int tj = tt - ti * (ti + 1) / 2;
+        const int c0 = tj * TR + (t - tt * G) * cw, r = ti * TR + lane;
+        if (c0 >= m) continue;
+        if (ti == tj) ht_task<R, C, RPL, true>(a22, ld, m, vS, yS, r, c0, cw, lane);
+        else ht_task<R, C, RPL, false>(a22, ld, m, vS, yS, r, c0, cw, lane);
     }
-    for (;;) {
-        ++nchunks;
-        // next chunk: the rest of this task, else the next valid task
-        int hn = h, r0n = r0 + HT_CH;
-        HtTask tn = t;
-        if (r0n >= t.rend) {
-            hn = h + NW;
-            while (hn < nh && !ht_task(hn, nloc, rank, CL, m, tn)) hn += NW;
-            r0n = tn.rbeg;
-        }
-        const bool more = hn < nh;
-        if (more) {
-            ht_issue(a22, ld, tn, r0n, stg + (buf ^ 1) * HT_STAGE_ELEMS, lane);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncwarp();
-        const float2* sb = stg + buf * HT_STAGE_ELEMS;
-        const bool diag = r0 < t.c0 + 8;  // the chunk holds the diagonal entries of the block
-#pragma unroll
-        for (int hf = 0; hf < HT_CH / 32; ++hf) {
-            const int r = r0 + lane + 32 * hf;
-            float2 a[8];
-#pragma unroll
-            for (int jj = 0; jj < 8; ++jj) a[jj] = sb[jj * HT_CH + lane + 32 * hf];  // 0 where not loaded
-            const float2 vr = (r < t.rend) ? vS[r] : czero<float2>();
-            float2 ra = czero<float2>();
-            const float2 vrx = make_float2(vr.x, vr.x), vry = make_float2(vr.y, vr.y);
-            if (!diag) {
-                float2 r1 = make_float2(0.f, 0.f), r2 = r1;
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    r1 = __ffma2_rn(a[jj], vxx[jj], r1);
-                    r2 = __ffma2_rn(a[jj], vyy[jj], r2);
-                    c1[jj] = __ffma2_rn(a[jj], vrx, c1[jj]);
-                    c2[jj] = __ffma2_rn(a[jj], vry, c2[jj]);
-                }
-                ra = make_float2(r1.x - r2.y, r1.y + r2.x);
-            } else {
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    const int c = t.c0 + jj;
-                    if (r > c) {
-                        ra = ra + a[jj] * v[jj];
-                        c1[jj] = __ffma2_rn(a[jj], vrx, c1[jj]);
-                        c2[jj] = __ffma2_rn(a[jj], vry, c2[jj]);
-                    } else if (r == c) {
-                        ra = ra + a[jj].x * v[jj];
-                    }
-                }
-            }
-            if (r < t.rend) atomic_add_c(&yS[r], ra);
-        }
-        __syncwarp();  // every lane is done with this stage before it is refilled
-        if (hn != h || !more) {  // the task is complete: add its column part
-#pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-                // conj(a) vr summed: (c1.x + c2.y, c2.x - c1.y)
-                const float sx = warp_sum(c1[jj].x + c2[jj].y), sy = warp_sum(c2[jj].x - c1[jj].y);
-                if (lane == 0 && jj < t.nc) atomic_add_c(&yS[t.c0 + jj], mk(sx, sy));
-                c1[jj] = c2[jj] = czero<float2>();
-            }
-            if (!more) break;
-#pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-                v[jj] = (jj < tn.nc) ? vS[tn.c0 + jj] : czero<float2>();
-                vxx[jj] = make_float2(v[jj].x, v[jj].x);
-                vyy[jj] = make_float2(v[jj].y, v[jj].y);
-            }
-        }
-        h = hn;
-        t = tn;
-        r0 = r0n;
-        buf ^= 1;
-    }
-    return nchunks;
 }
 
 // ------------------------------------------------------------------ trailing update, tensor cores
@@ -458,19 +433,23 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
         double* __restrict__ evec, typename Cx<R>::T* __restrict__ taupool, int nmax,
         int* __restrict__ status) {
     static_assert(!TC || sizeof(R) == 4, "tensor-core trailing update on the FP32 path only");
+    static_assert(MMF_NB <= 2 * (HT_THREADS / 32), "two columns of the panel per warp");
     typedef typename Cx<R>::T C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t tc_bar[3];
     __shared__ uint32_t tc_tmem;
-    C* vS = reinterpret_cast<C*>(smem_raw);   // nmax
-    C* yS = vS + nmax;                          // nmax: this CTA's partial y = A22 v
-    C* yF = yS + nmax;                          // nmax: full y (CL = 2)
-    C* wk = yF + nmax;                          // MMF_NB
-    C* vk = wk + MMF_NB;                        // MMF_NB
-    C* xw = vk + MMF_NB;                        // MMF_NB
-    C* xv = xw + MMF_NB;                        // MMF_NB
+    // x, then v: the partners push the next column into one buffer while this CTA still reads the other
+    C* vBuf = reinterpret_cast<C*>(smem_raw);  // 2 x nmax
+    C* yS = vBuf + 2 * (size_t)nmax;            // nmax: this CTA's partial y = A22 v, then its rows of w
+    C* wk = yS + nmax;                          // MMF_NB: row k of W, then W^H v
+    C* vk = wk + MMF_NB;                        // MMF_NB: row k of V, then V^H v
+    C* xw = vk + MMF_NB;                        // MMF_NB: this CTA's part of W^H v
+    C* xv = xw + MMF_NB;                        // MMF_NB: this CTA's part of V^H v
     C* sc = xv + MMF_NB;                        // 4 scalars: tau, scale, alpha2
-    R* red = reinterpret_cast<R*>(sc + 4);      // 66 (two block sums at once)
+    R* red = reinterpret_cast<R*>(sc + 4);      // 72: 0-15, 32, 33-48, 65 block sums; the rest is pushed
+    R* nrmP = red + 16;                         // by the partners: parts of ||x||^2 (8),
+    R* dotP = red + 49;                         // parts of w^H v (8 complex),
+    R* wnxt = red + 66;                         // w at row k + 1 before its last correction (complex)
     // one region shared by the her2k staging tiles and (FP32) the hemv's cp.async stages
     C* big = reinterpret_cast<C*>(smem_raw + ht_big_offset<R>(nmax));
     C* tVr = big;                               // MMF_NB x HT_TILE (her2k staging, transposed)
@@ -511,40 +490,88 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
         T.tmem = tc_tmem;
     }
 
+    // Rows in chunks of 32, chunk q with CTA q % CL.  In the O(m i) steps the warps split into CG
+    // groups over the panel's columns, each group's NCW warps over this CTA's chunks.
+    constexpr int CG = CL >= 6 ? 4 : CL >= 4 ? 2 : 1;
+    constexpr int NCW = (HT_THREADS / 32) / CG;
+    const int cw = warp % NCW, grp = warp / NCW;
+    C* pS = big;  // CG x (32 chunks of this CTA) partial sums (CG > 1)
+    C a2 = czero<C>();  // alpha2 of the previous column
     for (int j0 = 0; j0 < n; j0 += MMF_NB) {
         const int nb = min(MMF_NB, n - j0);
         for (int i = 0; i < nb; ++i) {
-            const int k = j0 + i;
-            // (a) pending panel updates of column k
-            if (i > 0) {
-                if (tid < i) {
-                    wk[tid] = conj(W[k + (int64_t)tid * ld]);
-                    vk[tid] = conj(V[k + (int64_t)tid * ld]);
+            const int k = j0 + i, m = n - k - 1;
+            C* vS = vBuf + (k & 1) * nmax;           // this column's x, then v, from row k + 1 on
+            const C* vP = vBuf + ((k & 1) ^ 1) * nmax;  // the previous column's v, from row k on
+            int q0 = k >> 5;                         // this CTA's first chunk with rows >= k
+            q0 += (rank - q0 % CL + CL) % CL;
+            const int nch = (n - 1) / 32 >= q0 ? ((n - 1) / 32 - q0) / CL + 1 : 0;
+            C* col = A + (int64_t)k * ld;
+            // (a) pending panel updates of column k; row k of the newest W is formed here
+            if (tid < i) {
+                wk[tid] = tid == i - 1 ? conj(mk(wnxt[0], wnxt[1]) + a2 * vP[0]) : conj(W[k + (int64_t)tid * ld]);
+                vk[tid] = tid == i - 1 ? conj(vP[0]) : conj(V[k + (int64_t)tid * ld]);
+            }
+            // (CG > 1: the column's entry this thread finishes below, loaded ahead)
+            C xpre = czero<C>();
+            if (CG > 1 && tid < nch * 32) {
+                const int r = (q0 + CL * (tid >> 5)) * 32 + (tid & 31);
+                if (r >= k && r < n) xpre = col[r];
+            }
+            __syncthreads();
+            R part = 0;
+            auto finish = [&](int r, C x0, C acc) {  // row r of the updated column
+                const C x = x0 - acc;
+                if (r == k) {
+                    dd[k] = (double)x.x;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < CL; ++q) (CL > 1 ? cluster.map_shared_rank(vS, q) : vS)[r - k - 1] = x;
+                    if (r >= k + 2) part += abs2(x);
                 }
-                __syncthreads();
-                for (int r = k + rank * HT_THREADS + tid; r < n; r += CL * HT_THREADS) {
-                    // unrolled so that the panel's loads (L2 latency each) are in flight together
-                    C acc = czero<C>(), acc2 = czero<C>();
+            };
+            for (int t = cw; t < nch; t += NCW) {
+                const int r = (q0 + CL * t) * 32 + lane;
+                // unrolled so that the panel's loads (L2 latency each) are in flight together
+                C acc = czero<C>(), acc2 = czero<C>();
+                if (r >= k && r < n) {
+                    const C x0 = CG == 1 ? col[r] : acc;
 #pragma unroll 8
-                    for (int c = 0; c < i; ++c) {
+                    for (int c = grp; c < i; c += CG) {
                         acc = acc + V[r + (int64_t)c * ld] * wk[c];
                         acc2 = acc2 + W[r + (int64_t)c * ld] * vk[c];
                     }
-                    A[r + (int64_t)k * ld] = A[r + (int64_t)k * ld] - (acc + acc2);
+                    if (CG == 1) finish(r, x0, acc + acc2);
                 }
-                if (CL > 1) cluster.sync(); else __syncthreads();
+                if (CG > 1) pS[(grp * nch + t) * 32 + lane] = acc + acc2;
             }
-            if (tid == 0 && rank == 0) dd[k] = (double)A[k + (int64_t)k * ld].x;
+            if (CG > 1) {
+                __syncthreads();
+                for (int o = tid; o < nch * 32; o += HT_THREADS) {
+                    const int r = (q0 + CL * (o >> 5)) * 32 + (o & 31);
+                    if (r < k || r >= n) continue;
+                    C acc = pS[o];
+#pragma unroll
+                    for (int q = 1; q < CG; ++q) acc = acc + pS[q * nch * 32 + o];
+                    finish(r, o == tid ? xpre : col[r], acc);
+                }
+            }
             if (k == n - 1) break;
-            const int m = n - k - 1;
-            C* col = A + (int64_t)k * ld;
 
-            // (b) reflector
-            R part = 0;
-            for (int r = k + 2 + tid; r < n; r += HT_THREADS) part += abs2(col[r]);
-            const R xn2 = block_sum(part, red);
+            // (b) reflector, the same in every CTA
+            const R xpart = block_sum(part, red);
+            if (CL > 1) {
+                if (tid < CL) cluster.map_shared_rank(nrmP, tid)[rank] = xpart;
+                cluster.sync();
+            }
             if (tid == 0) {
-                C alpha = col[k + 1];
+                R xn2 = xpart;
+                if (CL > 1) {
+                    xn2 = nrmP[0];
+#pragma unroll
+                    for (int q = 1; q < CL; ++q) xn2 += nrmP[q];
+                }
+                const C alpha = vS[0];
                 C t, s;
                 R beta;
                 if (xn2 == R(0) && alpha.y == R(0)) {
@@ -567,173 +594,134 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
             }
             __syncthreads();
             const C tk = sc[0], scale = sc[1];
-            for (int r = tid; r < n; r += HT_THREADS) {
-                C v;
-                if (r <= k) {
-                    v = czero<C>();
-                } else if (r == k + 1) {
-                    v = mk(R(1), R(0));
-                } else {
-                    v = col[r] * scale;
-                    if (CL == 1) col[r] = v;  // with a partner CTA still reading col, stored below
+            for (int rp = tid; rp < m; rp += HT_THREADS) {
+                const C v = rp == 0 ? mk(R(1), R(0)) : vS[rp] * scale;
+                const int r = rp + k + 1;
+                vS[rp] = v;
+                yS[rp] = czero<C>();
+                if (CL == 1 || (r >> 5) % CL == rank) {
+                    V[r + (int64_t)i * ld] = v;
+                    if (rp > 0) col[r] = v;
                 }
-                if (r > k) {
-                    vS[r - k - 1] = v;
-                    yS[r - k - 1] = czero<C>();
-                }
-                if (rank == 0) V[r + (int64_t)i * ld] = v;
             }
             __syncthreads();
 
-            // (c) y = A22 v (lower triangle) and (d) x_w = W^H v, x_v = V^H v
+            // (c) y = A22 v (lower triangle; this CTA's share) and (d) x_w = W^H v, x_v = V^H v (its rows)
             const C* a22 = A + (k + 1) + (int64_t)(k + 1) * ld;
-            // Tasks: the 2i dot products (every CTA needs them all), then this CTA's share of the
-            // hemv: column blocks of 8 (blocks rank, rank + CL, ...) cut into row segments of
-            // HT_SEG rows, so that tasks cost about the same and every warp gets some.
-            const int nblk = (m + 7) >> 3;
-            const int nloc = (nblk - rank + CL - 1) / CL;
-            const int nseg = (m + HT_SEG - 1) / HT_SEG;
-            const int ntask = 2 * i + nloc * nseg;
-            if constexpr (sizeof(R) == 4) {
-                for (int task = warp; task < 2 * i; task += NW) {
-                    const int c = task >> 1;
-                    const C* P = (task & 1) ? V : W;
-                    // unrolled: the loads of the V / W column are independent (L2 latency each)
-                    C acc = czero<C>(), acc2 = czero<C>();
-#pragma unroll 4
-                    for (int rp = lane; rp < m; rp += 64) {
-                        acc = acc + cmulc(P[(k + 1 + rp) + (int64_t)c * ld], vS[rp]);
-                        if (rp + 32 < m) acc2 = acc2 + cmulc(P[(k + 1 + rp + 32) + (int64_t)c * ld], vS[rp + 32]);
-                    }
-                    acc = acc + acc2;
-                    acc.x = warp_sum(acc.x);
-                    acc.y = warp_sum(acc.y);
-                    if (lane == 0) ((task & 1) ? xv : xw)[c] = acc;
-                }
-                (void)hemv_f32_staged(reinterpret_cast<const float2*>(a22), ld, m, reinterpret_cast<const float2*>(vS),
-                                reinterpret_cast<float2*>(yS),
-                                reinterpret_cast<float2*>(big) + (size_t)warp * 2 * HT_STAGE_ELEMS, rank, CL,
-                                nloc, nseg, warp, lane);
-            } else
-            for (int task = warp; task < ntask; task += NW) {
-                if (task < 2 * i) {
-                    const int c = task >> 1;
-                    const C* P = (task & 1) ? V : W;
-                    // unrolled: the loads of the V / W column are independent (L2 latency each)
-                    C acc = czero<C>(), acc2 = czero<C>();
-#pragma unroll 4
-                    for (int rp = lane; rp < m; rp += 64) {
-                        acc = acc + cmulc(P[(k + 1 + rp) + (int64_t)c * ld], vS[rp]);
-                        if (rp + 32 < m) acc2 = acc2 + cmulc(P[(k + 1 + rp + 32) + (int64_t)c * ld], vS[rp + 32]);
-                    }
-                    acc = acc + acc2;
-                    acc.x = warp_sum(acc.x);
-                    acc.y = warp_sum(acc.y);
-                    if (lane == 0) ((task & 1) ? xv : xw)[c] = acc;
-                    continue;
-                }
-                const int t = task - 2 * i;
-                const int q = t % nloc, sg = t / nloc;
-                const int c0 = (rank + CL * q) << 3;
-                const int rbeg = c0 + sg * HT_SEG;
-                if (rbeg >= m) continue;  // the segment lies below the matrix
-                const int rend = min(rbeg + HT_SEG, m);
-                const int nc = min(8, m - c0);
-                // v of the block's columns is read from shared memory at each use (registers go
-                // to the loads in flight)
-                C ca[8];
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) ca[jj] = czero<C>();
-                int r0 = rbeg;
-                if (sg == 0) {  // diagonal chunk (rows c0 .. c0+31)
-                    const int r = c0 + lane;
-                    if (r < m) {
-                        const C vr = vS[r];
-                        C ra = czero<C>();
-#pragma unroll
-                        for (int jj = 0; jj < 8; ++jj) {
-                            const int c = c0 + jj;
-                            if (jj < nc) {
-                                if (r > c) {
-                                    C a = a22[r + (int64_t)c * ld];
-                                    ra = ra + a * vS[c];
-                                    ca[jj] = ca[jj] + cmulc(a, vr);
-                                } else if (r == c) {
-                                    ra = ra + a22[r + (int64_t)c * ld].x * vS[c];
-                                }
-                            }
-                        }
-                        atomic_add_c(&yS[r], ra);
-                    }
-                    r0 = c0 + 32;
-                }
-                // strictly-lower chunks of 32 rows (this loop serves the FP64 path, which is bound by
-                // the FP64 units; the FP32 path streams through hemv_f32_staged)
-                for (; r0 < rend; r0 += 32) {
-                    const int rr = r0 + lane;
-                    if (rr < rend) {
-                        C a[8];
-#pragma unroll
-                        for (int jj = 0; jj < 8; ++jj)
-                            a[jj] = (jj < nc) ? a22[rr + (int64_t)(c0 + jj) * ld] : czero<C>();
-                        const C vr = vS[rr];
-                        C sa = czero<C>();
-#pragma unroll
-                        for (int jj = 0; jj < 8; ++jj) {
-                            const C v = (jj < nc) ? vS[c0 + jj] : czero<C>();
-                            sa = sa + a[jj] * v;
-                            ca[jj] = ca[jj] + cmulc(a[jj], vr);
-                        }
-                        atomic_add_c(&yS[rr], sa);
+            if (warp < i) {  // columns warp and warp + 16 of both matrices: all loads in flight together
+                const int ca = warp, cb = warp + NW < i ? warp + NW : warp;
+                const C *Wa = W + (int64_t)ca * ld, *Va = V + (int64_t)ca * ld, *Wb = W + (int64_t)cb * ld,
+                        *Vb = V + (int64_t)cb * ld;
+                C s0 = czero<C>(), s1 = s0, s2 = s0, s3 = s0;
+#pragma unroll 2
+                for (int t = 0; t < nch; ++t) {
+                    const int r = (q0 + CL * t) * 32 + lane;
+                    if (r > k && r < n) {
+                        const C v = vS[r - k - 1];
+                        s0 = s0 + cmulc(Wa[r], v);
+                        s1 = s1 + cmulc(Va[r], v);
+                        s2 = s2 + cmulc(Wb[r], v);
+                        s3 = s3 + cmulc(Vb[r], v);
                     }
                 }
 #pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    R sx = warp_sum(ca[jj].x), sy = warp_sum(ca[jj].y);
-                    if (lane == 0 && jj < nc) atomic_add_c(&yS[c0 + jj], mk(sx, sy));
+                for (int o = 16; o > 0; o >>= 1) {
+                    s0 = s0 + mk(__shfl_xor_sync(0xffffffffu, s0.x, o), __shfl_xor_sync(0xffffffffu, s0.y, o));
+                    s1 = s1 + mk(__shfl_xor_sync(0xffffffffu, s1.x, o), __shfl_xor_sync(0xffffffffu, s1.y, o));
+                    s2 = s2 + mk(__shfl_xor_sync(0xffffffffu, s2.x, o), __shfl_xor_sync(0xffffffffu, s2.y, o));
+                    s3 = s3 + mk(__shfl_xor_sync(0xffffffffu, s3.x, o), __shfl_xor_sync(0xffffffffu, s3.y, o));
+                }
+                if (lane == 0) {
+                    xw[ca] = s0;
+                    xv[ca] = s1;
+                    xw[cb] = s2;
+                    xv[cb] = s3;
                 }
             }
-            if (CL > 1) {
-                cluster.sync();  // both partial y complete
-                const C* yP = cluster.map_shared_rank(yS, rank ^ 1);
-                for (int rp = tid; rp < m; rp += HT_THREADS) yF[rp] = yS[rp] + yP[rp];
-                __syncthreads();
-            } else {
-                __syncthreads();  // y complete
+            ht_hemv<R, C>(a22, ld, m, vS, yS, warp * CL + rank, NW * CL, lane);
+            if (CL > 1) cluster.sync(); else __syncthreads();  // every part of y, x_w and x_v complete
+            for (int e = tid; e < 2 * i; e += HT_THREADS) {
+                const int c = e >> 1;
+                C* src = (e & 1) ? xv : xw;
+                C acc = src[c];
+                if (CL > 1) {
+                    acc = cluster.map_shared_rank(src, 0)[c];
+#pragma unroll
+                    for (int q = 1; q < CL; ++q) acc = acc + cluster.map_shared_rank(src, q)[c];
+                }
+                ((e & 1) ? vk : wk)[c] = acc;
             }
-            const C* yT = (CL > 1) ? yF : yS;
+            __syncthreads();
 
-            // (d) corrections, (e) w = tau y - (1/2) tau (w^H v) v
+            // (d) corrections, (e) w = tau y - (1/2) tau (w^H v) v, on this CTA's rows
             C dpart = czero<C>();
-            for (int rp = tid; rp < m; rp += HT_THREADS) {
-                C y = yT[rp], y2 = czero<C>();
-#pragma unroll 8
-                for (int c = 0; c < i; ++c) {
-                    y = y - V[(k + 1 + rp) + (int64_t)c * ld] * xw[c];
-                    y2 = y2 + W[(k + 1 + rp) + (int64_t)c * ld] * xv[c];
+            auto form_w = [&](int rp, C corr) {
+                C y = yS[rp];
+                if (CL > 1) {
+                    y = cluster.map_shared_rank(yS, 0)[rp];
+#pragma unroll
+                    for (int q = 1; q < CL; ++q) y = y + cluster.map_shared_rank(yS, q)[rp];
                 }
-                y = y - y2;
-                C w = tk * y;
-                yF[rp] = w;
+                const C w = tk * (y - corr);
+                yS[rp] = w;  // (the partners read only their own rows of this CTA's part)
                 dpart = dpart + cmulc(w, vS[rp]);
+                if (rp == 0) {
+#pragma unroll
+                    for (int q = 0; q < CL; ++q) {
+                        R* pn = CL > 1 ? cluster.map_shared_rank(wnxt, q) : wnxt;
+                        pn[0] = w.x;
+                        pn[1] = w.y;
+                    }
+                }
+            };
+            for (int t = cw; t < nch; t += NCW) {
+                const int r = (q0 + CL * t) * 32 + lane;
+                C acc = czero<C>(), acc2 = czero<C>();
+                if (r > k && r < n) {
+#pragma unroll 8
+                    for (int c = grp; c < i; c += CG) {
+                        acc = acc + V[r + (int64_t)c * ld] * wk[c];
+                        acc2 = acc2 + W[r + (int64_t)c * ld] * vk[c];
+                    }
+                    if (CG == 1) form_w(r - k - 1, acc + acc2);
+                }
+                if (CG > 1) pS[(grp * nch + t) * 32 + lane] = acc + acc2;
+            }
+            if (CG > 1) {
+                __syncthreads();
+                for (int o = tid; o < nch * 32; o += HT_THREADS) {
+                    const int r = (q0 + CL * (o >> 5)) * 32 + (o & 31);
+                    if (r <= k || r >= n) continue;
+                    C acc = pS[o];
+#pragma unroll
+                    for (int q = 1; q < CG; ++q) acc = acc + pS[q * nch * 32 + o];
+                    form_w(r - k - 1, acc);
+                }
             }
             R dx, dy;
             block_sum2(dpart.x, dpart.y, red, dx, dy);
-            const C alpha2 = R(-0.5) * (tk * mk(dx, dy));
-            if (rank == 0)
-                for (int r = tid; r < n; r += HT_THREADS) {
-                    C w = czero<C>();
-                    if (r > k) w = yF[r - k - 1] + alpha2 * vS[r - k - 1];
-                    W[r + (int64_t)i * ld] = w;
-                }
             if (CL > 1) {
-                cluster.sync();  // both CTAs are done with column k
-                if (rank == 0)
-                    for (int r = k + 2 + tid; r < n; r += HT_THREADS) col[r] = vS[r - k - 1];
-            } else {
-                __syncthreads();
+                if (tid < CL) {
+                    R* pd = cluster.map_shared_rank(dotP, tid);
+                    pd[2 * rank] = dx;
+                    pd[2 * rank + 1] = dy;
+                }
+                cluster.sync();
+                dx = dotP[0];
+                dy = dotP[1];
+#pragma unroll
+                for (int q = 1; q < CL; ++q) {
+                    dx += dotP[2 * q];
+                    dy += dotP[2 * q + 1];
+                }
+            }
+            a2 = R(-0.5) * (tk * mk(dx, dy));
+            for (int o = tid; o < nch * 32; o += HT_THREADS) {
+                const int r = (q0 + CL * (o >> 5)) * 32 + (o & 31);
+                if (r > k && r < n) W[r + (int64_t)i * ld] = yS[r - k - 1] + a2 * vS[r - k - 1];
             }
         }
+        if (CL > 1) cluster.sync(); else __syncthreads();  // the panel is complete
 
         // trailing her2k on the lower triangle of A(c0:, c0:)
         const int c0 = j0 + nb;
@@ -811,6 +799,7 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
             if (CL > 1) cluster.sync();
         }
     }
+    if (CL > 1) cluster.sync();  // no CTA leaves while a partner may still read its shared memory
     if constexpr (TC) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -835,9 +824,10 @@ int mmf_hetrd_max_n(int fp32) {
     return (int)((227 * 1024 - fixed - 64) / (3 * cs));
 }
 
+// CL CTAs per system; *fits (if given) only reports whether one wave holds all the clusters.
 template <class R, int CL, bool TC>
-static cudaError_t launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
-                                double* evec, void* tau, size_t sm, int* status) {
+static cudaError_t launch_hetrd_cl(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
+                                   double* evec, void* tau, size_t sm, int* status, bool* fits) {
     typedef typename Cx<R>::T C;
     cudaError_t err = cudaFuncSetAttribute(k_hetrd<R, CL, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
@@ -853,8 +843,43 @@ static cudaError_t launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (fits) {
+        int nc = 0;
+        err = cudaOccupancyMaxActiveClusters(&nc, k_hetrd<R, CL, TC>, &cfg);
+        *fits = err == cudaSuccess && L.count <= nc;
+        return err;
+    }
     return cudaLaunchKernelEx(&cfg, k_hetrd<R, CL, TC>, L.desc, L.idx, (C*)H, (C*)Vp, (C*)Wp, dvec, evec,
                               (C*)tau, L.nmax, status);
+}
+
+// The most CTAs per system that run in one wave (a GB300 holds 15 clusters of 8, 23 of 6, 36 of 4);
+// from 4 on only for systems long enough that each CTA keeps a few row chunks (the barriers of a larger
+// cluster cost more than a small column's work).
+template <class R, bool TC>
+static cudaError_t launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
+                                double* evec, void* tau, size_t sm, int* status) {
+    bool fits = false;
+    cudaError_t e;
+    if (L.nmax >= HT_CL8_N) {
+        e = launch_hetrd_cl<R, 8, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_hetrd_cl<R, 8, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+    }
+    if (L.nmax >= HT_CL8_N) {
+        e = launch_hetrd_cl<R, 6, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_hetrd_cl<R, 6, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+    }
+    if (L.nmax >= HT_CL4_N) {
+        e = launch_hetrd_cl<R, 4, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
+        if (e != cudaSuccess) return e;
+        if (fits) return launch_hetrd_cl<R, 4, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+    }
+    e = launch_hetrd_cl<R, 2, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
+    if (e != cudaSuccess) return e;
+    if (fits) return launch_hetrd_cl<R, 2, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+    return launch_hetrd_cl<R, 1, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
 }
 
 cudaError_t mmf_launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
@@ -862,19 +887,9 @@ cudaError_t mmf_launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, do
     if (L.count <= 0) return cudaSuccess;
     if (L.nmax > mmf_hetrd_max_n(fp32)) return cudaErrorInvalidValue;
     const size_t sm = hetrd_smem(L.nmax, fp32);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // two CTAs per system while that still fits the GPU in one wave
-    const bool pair = 2 * L.count <= sms;
-    if (fp32 && tc)
-        return pair ? launch_hetrd<float, 2, true>(L, H, Vp, Wp, dvec, evec, tau, sm, status)
-                    : launch_hetrd<float, 1, true>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
-    if (fp32)
-        return pair ? launch_hetrd<float, 2, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status)
-                    : launch_hetrd<float, 1, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
-    return pair ? launch_hetrd<double, 2, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status)
-                : launch_hetrd<double, 1, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
+    if (fp32 && tc) return launch_hetrd<float, true>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
+    if (fp32) return launch_hetrd<float, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
+    return launch_hetrd<double, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
 }
 
 // ------------------------------------------------------------------ self-test
