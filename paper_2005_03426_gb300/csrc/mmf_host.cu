@@ -153,6 +153,9 @@ struct mmf_batch {
     // per-stage CUDA-event timing (optional)
     int timing_runs = 0, runs_recorded = 0;
     std::vector<cudaEvent_t> ev;
+    // side streams for the solver paths of a mixed batch (run_branches); empty if it has one path
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> side_ev;  // side_ev[i]: end of side[i]'s branch; the last one: the fork
     // CUDA graph of the whole run (optional)
     bool use_graph = false;
     cudaGraphExec_t graph_exec = nullptr;
@@ -494,7 +497,15 @@ static void fill_coef(const mmf_batch* b, double2* dst) {
     }
 }
 
+static void drop_side_streams(mmf_batch* b) {
+    for (cudaEvent_t e : b->side_ev) cudaEventDestroy(e);
+    for (cudaStream_t st : b->side) cudaStreamDestroy(st);
+    b->side_ev.clear();
+    b->side.clear();
+}
+
 static void free_batch_memory(mmf_batch* b) {
+    drop_side_streams(b);  // (their last work was joined into the batch's stream)
     if (b->base) {
         cudaFreeAsync(b->base, b->stream);
         b->ctx->used -= b->bytes;
@@ -854,6 +865,26 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
         delete b;
         return fail(MMF_ERR_CUDA, std::string("upload: ") + cudaGetErrorString(e));
     }
+    // a side stream for each solver path of the reduction or the back-transform beyond the first
+    int nred = !b->medium.empty() + !b->tiny.empty(), nback = !b->bts.empty() + !b->btc.empty();
+    for (int ci = 0; ci < 4; ++ci) nred += !b->sbr[ci].empty();
+    for (int ci = 0; ci < 5; ++ci) nback += !b->sbt[ci].empty();
+    const int nside = std::max(nred, nback) - 1;
+    for (int i = 0; i < nside && e == cudaSuccess; ++i) {
+        cudaStream_t ss = nullptr;
+        e = cudaStreamCreateWithFlags(&ss, cudaStreamNonBlocking);
+        if (e == cudaSuccess) b->side.push_back(ss);
+    }
+    for (int i = 0; i <= nside && nside > 0 && e == cudaSuccess; ++i) {
+        cudaEvent_t ev = nullptr;
+        e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) b->side_ev.push_back(ev);
+    }
+    if (e != cudaSuccess) {
+        free_batch_memory(b);
+        delete b;
+        return fail(MMF_ERR_CUDA, std::string("side streams: ") + cudaGetErrorString(e));
+    }
     *out = b;
     return MMF_OK;
 }
@@ -984,6 +1015,83 @@ static cudaError_t refine_gram(mmf_batch* b, const MmfLaunch& L, int second) {
     return mmf_launch_refine_gram(L, b->d_X1, b->d_R, b->d_T, second);
 }
 
+// Independent launches of one stage, one per solver path, side by side: the paths work on different
+// systems, and each leaves SMs idle (a chase or a small reduction is a few long-running CTAs), so that
+// run one after another they add up where together they take about the longest (uneven batch of 256,
+// mixed: reductions 132 -> 88 ms, back-transforms 58 -> 33).  The first branch runs on the batch's stream, the others on its side
+// streams between a fork event and join events, so whatever follows on the batch's stream (frees and
+// other streams' waits included) is ordered after all of them, also when a launch fails.
+struct Branches {
+    mmf_batch* b;
+    int used = 0;
+    cudaError_t err = cudaSuccess;
+    explicit Branches(mmf_batch* b_) : b(b_) {
+        if (!b->side.empty()) err = cudaEventRecord(b->side_ev.back(), b->stream);
+    }
+    cudaStream_t next() {
+        const int i = used++;
+        if (i == 0) return b->stream;
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(b->side[i - 1], b->side_ev.back(), 0);
+        return b->side[i - 1];
+    }
+    cudaError_t join() {
+        for (int i = 0; i + 1 < used; ++i) {
+            cudaError_t e = cudaEventRecord(b->side_ev[i], b->side[i]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->side_ev[i], 0);
+            if (err == cudaSuccess) err = e;
+        }
+        return err;
+    }
+};
+
+static MmfLaunch on_stream(MmfLaunch L, cudaStream_t st) {
+    L.stream = st;
+    return L;
+}
+
+static int launch_reductions(mmf_batch* b, Branches& br, int fp32) {
+    if (!b->medium.empty()) {
+        MmfLaunch Lm = on_stream(launch_of(b, b->medium, b->d_medium, b->nmax_medium), br.next());
+        LAUNCH(mmf_launch_hetrd(Lm, b->d_H, b->d_Vp, b->d_Wp, b->d_d, b->d_e, b->d_tau, fp32, b->hetrd_tc, b->d_status),
+               1);
+    }
+    for (int ci = 3; ci >= 0; --ci) {  // banded systems: bulge chase, the widest bands first
+        if (b->sbr[ci].empty()) continue;
+        MmfLaunch Lb = on_stream(launch_of(b, b->sbr[ci], b->d_sbr[ci], b->nmax_sbr[ci]), br.next());
+        LAUNCH(mmf_launch_sbr_chase(Lb, 8 << ci, b->d_H, b->d_Zf, b->d_d, b->d_e, b->d_status, fp32), 1);
+    }
+    if (!b->tiny.empty()) {
+        MmfLaunch Lt = on_stream(launch_of(b, b->tiny, b->d_tiny, b->nmax_tiny), br.next());
+        LAUNCH(mmf_launch_hetrd_small(Lt, b->d_H, b->d_d, b->d_e, b->d_tau, fp32), 1);
+    }
+    return MMF_OK;
+}
+
+static int launch_backtransforms(mmf_batch* b, Branches& br, int fp32) {
+    if (!b->sbt[4].empty()) {  // banded systems on the tensor cores (T factors, products, transpose)
+        MmfLaunch Lt = on_stream(launch_of(b, b->sbt[4], b->d_sbt[4], b->nmax_sbt[4]), br.next());
+        LAUNCH(mmf_launch_sbr_bt_tc(Lt, b->d_Zf, b->d_Y, b->d_work, b->d_oz, (float2*)b->d_Zp, b->d_status), 3);
+    }
+    for (int ci = 3; ci >= 0; --ci) {  // banded systems: Z = Q Y from the chase's reflectors
+        if (b->sbt[ci].empty()) continue;
+        MmfLaunch Lb = on_stream(launch_of(b, b->sbt[ci], b->d_sbt[ci], b->nmax_sbt[ci]), br.next());
+        LAUNCH(mmf_launch_sbr_bt(Lb, 8 << ci, b->d_Zf, b->d_Y, b->d_work, b->d_Zp, fp32), 2);
+    }
+    if (!b->btc.empty()) {
+        MmfLaunch Lc = on_stream(launch_of(b, b->btc, b->d_btc, b->nmax_btc), br.next());
+        int nl = 0;
+        LAUNCH(mmf_launch_backtransform_tc(Lc, b->btc_n.data(), b->d_H, b->d_tau, b->d_Y, b->d_Zp, b->d_oz, b->d_btjobs,
+                                           b->d_status, &nl),
+               0);
+        g_launches += nl;
+    }
+    if (!b->bts.empty()) {
+        MmfLaunch Ls = on_stream(launch_of(b, b->bts, b->d_bts, b->nmax_bts), br.next());
+        LAUNCH(mmf_launch_backtransform(Ls, b->d_H, b->d_tau, b->d_Vp, b->d_Y, b->d_Zp, fp32), 2);
+    }
+    return MMF_OK;
+}
+
 static int stage_eig(mmf_batch* b) {
     const int fp32 = b->precision == MMF_MIXED;
     mark(b, ST_JACOBI);
@@ -994,20 +1102,11 @@ static int stage_eig(mmf_batch* b) {
     if (!b->large.empty()) {
         MmfLaunch Ll = launch_of(b, b->large, b->d_large, b->nmax_large);
         mark(b, ST_HETRD);
-        if (!b->medium.empty()) {
-            MmfLaunch Lm = launch_of(b, b->medium, b->d_medium, b->nmax_medium);
-            LAUNCH(mmf_launch_hetrd(Lm, b->d_H, b->d_Vp, b->d_Wp, b->d_d, b->d_e, b->d_tau, fp32, b->hetrd_tc,
-                                    b->d_status),
-                   1);
-        }
-        if (!b->tiny.empty()) {
-            MmfLaunch Lt = launch_of(b, b->tiny, b->d_tiny, b->nmax_tiny);
-            LAUNCH(mmf_launch_hetrd_small(Lt, b->d_H, b->d_d, b->d_e, b->d_tau, fp32), 1);
-        }
-        for (int ci = 0; ci < 4; ++ci) {  // banded systems: bulge chase
-            if (b->sbr[ci].empty()) continue;
-            MmfLaunch Lb = launch_of(b, b->sbr[ci], b->d_sbr[ci], b->nmax_sbr[ci]);
-            LAUNCH(mmf_launch_sbr_chase(Lb, 8 << ci, b->d_H, b->d_Zf, b->d_d, b->d_e, b->d_status, fp32), 1);
+        {
+            Branches br(b);
+            const int rc = launch_reductions(b, br, fp32);
+            CU(br.join());
+            if (rc != MMF_OK) return rc;
         }
         for (int i : b->huge) {  // one system at a time over the whole GPU
             const MmfDesc& d = b->desc[i];
@@ -1021,26 +1120,11 @@ static int stage_eig(mmf_batch* b) {
         LAUNCH(mmf_launch_tridiag_eig(Ll, b->d_d, b->d_e, b->d_aux, b->d_e2, b->d_E, b->d_Y, b->d_work,
                                       b->d_status, fp32, 3), 3);
         mark(b, ST_BACKTRANSFORM);
-        if (!b->bts.empty()) {
-            MmfLaunch Ls = launch_of(b, b->bts, b->d_bts, b->nmax_bts);
-            LAUNCH(mmf_launch_backtransform(Ls, b->d_H, b->d_tau, b->d_Vp, b->d_Y, b->d_Zp, fp32), 2);
-        }
-        if (!b->btc.empty()) {
-            MmfLaunch Lc = launch_of(b, b->btc, b->d_btc, b->nmax_btc);
-            int nl = 0;
-            LAUNCH(mmf_launch_backtransform_tc(Lc, b->btc_n.data(), b->d_H, b->d_tau, b->d_Y, b->d_Zp, b->d_oz,
-                                               b->d_btjobs, b->d_status, &nl),
-                   0);
-            g_launches += nl;
-        }
-        for (int ci = 0; ci < 4; ++ci) {  // banded systems: Z = Q Y from the chase's reflectors
-            if (b->sbt[ci].empty()) continue;
-            MmfLaunch Lb = launch_of(b, b->sbt[ci], b->d_sbt[ci], b->nmax_sbt[ci]);
-            LAUNCH(mmf_launch_sbr_bt(Lb, 8 << ci, b->d_Zf, b->d_Y, b->d_work, b->d_Zp, fp32), 2);
-        }
-        if (!b->sbt[4].empty()) {  // the same on the tensor cores (T factors, products, transpose)
-            MmfLaunch Lt = launch_of(b, b->sbt[4], b->d_sbt[4], b->nmax_sbt[4]);
-            LAUNCH(mmf_launch_sbr_bt_tc(Lt, b->d_Zf, b->d_Y, b->d_work, b->d_oz, (float2*)b->d_Zp, b->d_status), 3);
+        {
+            Branches br(b);
+            const int rc = launch_backtransforms(b, br, fp32);
+            CU(br.join());
+            if (rc != MMF_OK) return rc;
         }
         if (fp32) LAUNCH(mmf_launch_widen(Ll, b->d_Zp, b->d_Zf, fp32), 1);
     } else {
