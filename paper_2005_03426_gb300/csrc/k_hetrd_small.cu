@@ -141,6 +141,99 @@ k_hetrd_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, ty
     if (tid == 0) dd[n - 1] = (double)L[hs_at(n, n - 1, n - 1)].x;
 }
 
+// Back-transform Z = P_0 P_1 ... P_{n-2} Y of the same systems (S5): a CTA takes HS_BT_NC columns of
+// Z in shared memory and applies the reflectors one by one, last first, each column's rows dealt over
+// HS_BT_RG threads.  FP64-bound like the reduction (8 n^3 / 2 real flops a system), with two barriers a
+// reflector, where the blocked form's T factors and 64-row tiles cost more than they save at these
+// sizes: n = 82 in FP64, one system 0.27 ms (k_larft and k_backtransform 1.27), 200 systems
+// 1.8 ms (4.65).
+#define HS_BT_NC 16
+#define HS_BT_THREADS 128
+#define HS_BT_RG (HS_BT_THREADS / HS_BT_NC)
+
+template <class R>
+__global__ void __launch_bounds__(HS_BT_THREADS)
+k_bt_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, const typename Cx<R>::T* __restrict__ H,
+           const typename Cx<R>::T* __restrict__ taupool, const double* __restrict__ Yg,
+           typename Cx<R>::T* __restrict__ Zout) {
+    typedef typename Cx<R>::T C;
+    extern __shared__ __align__(16) unsigned char hs_smem[];
+    __shared__ C vs[2][HS_ROWS], red[HS_BT_THREADS / 32][HS_BT_NC];
+    C(*z)[HS_BT_NC] = reinterpret_cast<C(*)[HS_BT_NC]>(hs_smem);  // n x HS_BT_NC
+    const MmfDesc d = descs[idx[blockIdx.y]];
+    const int n = d.n, ld = d.ld;
+    const int c0 = blockIdx.x * HS_BT_NC;
+    if (c0 >= n) return;
+    const C* A = H + d.mat_off;
+    const C* tau = taupool + d.vec_off;
+    const double* Y = Yg + d.sq_off;
+    C* Z = Zout + d.mat_off;
+    const int tx = threadIdx.x, cl = tx % HS_BT_NC, g = tx / HS_BT_NC, warp = tx >> 5;
+    for (int r = g; r < n; r += HS_BT_RG)
+        z[r][cl] = mk(c0 + cl < n ? (R)Y[(int64_t)r * n + c0 + cl] : R(0), R(0));
+    // v of reflector k on rows k + 1 .. n - 1: 1, then A(k + 2 .., k)
+    if (tx == 0) vs[0][0] = mk(R(1), R(0));
+    C t = tau[n - 2];
+    __syncthreads();
+    int buf = 0;
+    for (int k = n - 2; k >= 0; --k) {
+        const int m = n - k - 1;
+        C v0 = czero<C>(), v1 = v0, tn = v0;  // the next reflector, loading meanwhile
+        if (k > 0) {
+            const C* a = A + (k + 1) + (int64_t)(k - 1) * ld;  // entry e of v, e >= 1, at a[e - 1]
+            if (tx < m) v0 = a[tx];
+            if (tx + HS_BT_THREADS < m) v1 = a[tx + HS_BT_THREADS];
+            tn = tau[k - 1];
+        }
+        const C* v = vs[buf];
+        C w = czero<C>(), w1 = w;
+        int i = g;
+        for (; i + HS_BT_RG < m; i += 2 * HS_BT_RG) {
+            w = w + cmulc(v[i], z[k + 1 + i][cl]);
+            w1 = w1 + cmulc(v[i + HS_BT_RG], z[k + 1 + i + HS_BT_RG][cl]);
+        }
+        if (i < m) w = w + cmulc(v[i], z[k + 1 + i][cl]);
+        w = w + w1;
+#pragma unroll
+        for (int o = HS_BT_NC; o < 32; o <<= 1) {
+            w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
+            w.y += __shfl_xor_sync(0xffffffffu, w.y, o);
+        }
+        if ((tx & 31) < HS_BT_NC) red[warp][cl] = w;
+        __syncthreads();
+        w = red[0][cl];
+#pragma unroll
+        for (int q = 1; q < HS_BT_THREADS / 32; ++q) w = w + red[q][cl];
+        const C tw = t * w;
+        for (int q = g; q < m; q += HS_BT_RG) z[k + 1 + q][cl] = z[k + 1 + q][cl] - tw * v[q];
+        if (k > 0) {
+            C* vn = vs[buf ^ 1];
+            if (tx == 0) vn[0] = mk(R(1), R(0));
+            if (tx < m) vn[tx + 1] = v0;
+            if (tx + HS_BT_THREADS < m) vn[tx + HS_BT_THREADS + 1] = v1;
+            t = tn;
+        }
+        __syncthreads();
+        buf ^= 1;
+    }
+    const int nc = min(HS_BT_NC, n - c0);
+    for (int e = tx; e < nc * n; e += HS_BT_THREADS) {
+        const int c = e / n, r = e - c * n;
+        Z[r + (int64_t)(c0 + c) * ld] = z[r][c];
+    }
+}
+
+template <class R>
+static cudaError_t launch_bt_small(const MmfLaunch& L, const void* H, const void* tau, const double* Y, void* Z) {
+    typedef typename Cx<R>::T C;
+    const size_t sm = sizeof(C) * HS_BT_NC * (size_t)L.nmax;
+    cudaError_t e = cudaFuncSetAttribute(k_bt_small<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_bt_small<R><<<dim3((L.nmax + HS_BT_NC - 1) / HS_BT_NC, L.count), HS_BT_THREADS, sm, L.stream>>>(
+        L.desc, L.idx, (const C*)H, (const C*)tau, Y, (C*)Z);
+    return cudaGetLastError();
+}
+
 template <class R>
 static cudaError_t launch_small(const MmfLaunch& L, void* H, double* dvec, double* evec, void* tau) {
     typedef typename Cx<R>::T C;
@@ -160,4 +253,10 @@ cudaError_t mmf_launch_hetrd_small(const MmfLaunch& L, void* H, double* dvec, do
     if (L.count <= 0) return cudaSuccess;
     if (L.nmax > mmf_hetrd_small_n(fp32)) return cudaErrorInvalidValue;
     return fp32 ? launch_small<float>(L, H, dvec, evec, tau) : launch_small<double>(L, H, dvec, evec, tau);
+}
+
+cudaError_t mmf_launch_bt_small(const MmfLaunch& L, const void* H, const void* tau, const double* Y, void* Z, int fp32) {
+    if (L.count <= 0) return cudaSuccess;
+    if (L.nmax > mmf_hetrd_small_n(fp32)) return cudaErrorInvalidValue;
+    return fp32 ? launch_bt_small<float>(L, H, tau, Y, Z) : launch_bt_small<double>(L, H, tau, Y, Z);
 }

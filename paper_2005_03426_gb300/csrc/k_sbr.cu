@@ -588,69 +588,98 @@ __global__ void __launch_bounds__(128) k_sbr_bt_f32(const MmfDesc* __restrict__ 
     }
 }
 
-// FP64: the same with the window in shared memory (a column per thread, BMAX rows).
-template <int BMAX>
+// FP64: the same with the window in shared memory; a CTA of 128 threads takes NC columns, each
+// column's window rows dealt over RG = 128 / NC threads.  The SM's FP64 units bound it (a warp-wide
+// FP64 instruction takes 64 cycles on its scheduler, 19 over the four): 8 n^3 flops per system at
+// least, which 8 systems of n = 1323 spread over the whole GPU do in 120 ms.  One column per thread
+// (128 columns per CTA) left 64 of 152 SMs idle there and took 417 ms; slabs of 32 and 16 columns keep
+// all four schedulers of a CTA's SM busy and spread evenly: 328 ms.  Rows past the band's b are
+// skipped.
+template <int BMAX, int NC>
 __global__ void __launch_bounds__(128) k_sbr_bt_f64(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                                                    const double2* __restrict__ store_base,
                                                    const double* __restrict__ Yg, double* __restrict__ work) {
-    extern __shared__ __align__(16) double2 sbt_smem[];
-    double2* vs = sbt_smem;                 // [2][BMAX]
-    double2* ts = vs + 2 * BMAX;            // [2]
-    double2* win = ts + 2;                  // [BMAX][128]
+    constexpr int RG = 128 / NC, WG = 32 / NC > 0 ? 32 / NC : 1, NP = RG / WG;  // row groups: all, per warp; partial sums
+    __shared__ double2 vs[2][BMAX], ts[2], red[NP][NC], win[BMAX][NC];
     const MmfDesc d = descs[idx[blockIdx.y]];
     const int n = d.n, b = d.band;
-    const int c = blockIdx.x * 128 + threadIdx.x;
-    if (blockIdx.x * 128 >= n) return;
+    if (blockIdx.x * NC >= n) return;
+    const int tx = threadIdx.x, cl = tx % NC, g = tx / NC, warp = tx >> 5;
+    const int c = blockIdx.x * NC + cl;
     const bool act = c < n;
     const double2* V = store_base + d.mat_off;
     const double2* T = V + sbr_nref(n, b) * b;
     const double* Y = Yg + d.sq_off;
     double2* Z = reinterpret_cast<double2*>(sbr_zbase(work, d));
-    const int tx = threadIdx.x;
-    if (act) Z[c] = make_double2(Y[c], 0.0);
+    const double2 z0 = make_double2(0.0, 0.0);
+    if (act && g == 0) Z[c] = make_double2(Y[c], 0.0);  // row 0: no reflector touches it
     const int np = sbr_passes(n, b);
     for (int s = 0; s < np; ++s) {
         const int jtop = n - 2 - s * b;
         const int64_t off = sbr_off(n, b, s);
-        int top = 0;  // window slot of the window's first row (circular)
-        for (int q = 0; q < BMAX; ++q) win[q * 128 + tx] = make_double2(0.0, 0.0);
-        if (act) win[tx] = s == 0 ? make_double2(Y[(int64_t)(n - 1) * n + c], 0.0) : Z[(int64_t)(n - 1) * n + c];
-        if (tx < BMAX) vs[tx] = tx < b ? V[(off + jtop) * b + tx] : make_double2(0.0, 0.0);
+        int top = 0;  // window slot of the window's first row (circular over b slots)
+        for (int q = g; q < b; q += RG) win[q][cl] = z0;
+        __syncthreads();
+        if (g == 0 && act)
+            win[0][cl] = s == 0 ? make_double2(Y[(int64_t)(n - 1) * n + c], 0.0) : Z[(int64_t)(n - 1) * n + c];
+        if (tx < b) vs[0][tx] = V[(off + jtop) * b + tx];
         if (tx == 0) ts[0] = T[off + jtop];
         __syncthreads();
         int buf = 0;
         for (int j = jtop; j >= 0; --j) {
-            double2 vn = make_double2(0.0, 0.0), tn = make_double2(0.0, 0.0);
+            double2 vn = z0, tn = z0, zn = z0;  // the next step's reflector and row, loading meanwhile
+            const int r = j + 1 + s * b;        // first row of the window
             if (j > 0) {
                 if (tx < b) vn = V[(off + j - 1) * b + tx];
                 if (tx == 0) tn = T[off + j - 1];
+                if (g == 0 && act)
+                    zn = s == 0 ? make_double2(Y[(int64_t)(r - 1) * n + c], 0.0) : Z[(int64_t)(r - 1) * n + c];
             }
-            const double2* vv = vs + buf * BMAX;
-            double2 w = make_double2(0.0, 0.0);
-            for (int q = 0; q < BMAX; ++q) w = w + cmulc(vv[q], win[((top + q) % BMAX) * 128 + tx]);
+            // w = v^H z over this thread's rows, then over the groups
+            double2 w = z0;
+            for (int q = g; q < b; q += RG) {
+                int sl = top + q;
+                sl -= sl >= b ? b : 0;
+                w = w + cmulc(vs[buf][q], win[sl][cl]);
+            }
+#pragma unroll
+            for (int o = NC; o < 32; o <<= 1) {
+                w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
+                w.y += __shfl_xor_sync(0xffffffffu, w.y, o);
+            }
+            if ((tx & 31) < NC) red[warp % NP][cl] = w;
+            __syncthreads();
+            w = red[0][cl];
+#pragma unroll
+            for (int q = 1; q < NP; ++q) w = w + red[q][cl];
             const double2 tw = ts[buf] * w;
-            for (int q = 0; q < BMAX; ++q) {
-                double2& z = win[((top + q) % BMAX) * 128 + tx];
-                z = z - tw * vv[q];
+            const int bot = top == 0 ? b - 1 : top - 1;  // slot of the window's last row, the one that leaves
+            for (int q = g; q < b; q += RG) {
+                int sl = top + q;
+                sl -= sl >= b ? b : 0;
+                const double2 z = win[sl][cl] - tw * vs[buf][q];
+                if (j > 0 && q == b - 1) {
+                    if (act && r + q < n) Z[(int64_t)(r + q) * n + c] = z;
+                } else {
+                    win[sl][cl] = z;
+                }
             }
             if (j > 0) {
-                const int r = j + 1 + s * b;
-                const int bot = (top + BMAX - 1) % BMAX;
-                if (act && r + BMAX - 1 < n) Z[(int64_t)(r + BMAX - 1) * n + c] = win[bot * 128 + tx];
-                top = bot;  // the slot of the leaving row takes the new first row
-                const int64_t row = r - 1;
-                win[top * 128 + tx] = act ? (s == 0 ? make_double2(Y[row * n + c], 0.0) : Z[row * n + c])
-                                          : make_double2(0.0, 0.0);
-                if (tx < BMAX) vs[(buf ^ 1) * BMAX + tx] = vn;
+                __syncthreads();  // the last row's slot has been read
+                if (g == 0) win[bot][cl] = zn;
+                top = bot;
+                if (tx < b) vs[buf ^ 1][tx] = vn;
                 if (tx == 0) ts[buf ^ 1] = tn;
             }
             __syncthreads();
             buf ^= 1;
         }
         const int r0 = 1 + s * b;
-        if (act)
-            for (int q = 0; q < BMAX; ++q)
-                if (r0 + q < n) Z[(int64_t)(r0 + q) * n + c] = win[((top + q) % BMAX) * 128 + tx];
+        for (int q = g; q < b; q += RG) {
+            int sl = top + q;
+            sl -= sl >= b ? b : 0;
+            if (act && r0 + q < n) Z[(int64_t)(r0 + q) * n + c] = win[sl][cl];
+        }
         __syncthreads();
     }
 }
@@ -743,15 +772,18 @@ static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, dou
 
 template <int BMAX>
 static cudaError_t launch_bt(const MmfLaunch& L, const double2* store, const double* Y, double* work, int fp32) {
-    dim3 g((L.nmax + 127) / 128, L.count);
     if (fp32) {
-        k_sbr_bt_f32<BMAX><<<g, 128, 0, L.stream>>>(L.desc, L.idx, store, Y, work);
-    } else {
-        const size_t sm = sizeof(double2) * (2 * BMAX + 2 + (size_t)BMAX * 128);
-        cudaError_t e = cudaFuncSetAttribute(k_sbr_bt_f64<BMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_sbr_bt_f64<BMAX><<<g, 128, sm, L.stream>>>(L.desc, L.idx, store, Y, work);
+        k_sbr_bt_f32<BMAX><<<dim3((L.nmax + 127) / 128, L.count), 128, 0, L.stream>>>(L.desc, L.idx, store, Y, work);
+        return cudaGetLastError();
     }
+    // 32 columns per CTA once that gives every SM several CTAs (fewer exchanges per column), else 16
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if ((int64_t)((L.nmax + 31) / 32) * L.count >= 8 * (int64_t)sms)
+        k_sbr_bt_f64<BMAX, 32><<<dim3((L.nmax + 31) / 32, L.count), 128, 0, L.stream>>>(L.desc, L.idx, store, Y, work);
+    else
+        k_sbr_bt_f64<BMAX, 16><<<dim3((L.nmax + 15) / 16, L.count), 128, 0, L.stream>>>(L.desc, L.idx, store, Y, work);
     return cudaGetLastError();
 }
 

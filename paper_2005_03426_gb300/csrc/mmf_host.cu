@@ -100,10 +100,10 @@ struct mmf_batch {
     int nmax_sbt[5] = {0, 0, 0, 0, 0};
     int* d_sbt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     std::vector<int> rband, rfull;                     // mixed: hybrid / full second refinement step
-    std::vector<int> btc, bts;                         // large: back-transform on tensor cores / SIMT
+    std::vector<int> btc, bts, btt;                    // large: back-transform on tensor cores / SIMT / one CTA's columns
     std::vector<int> btc_n;                            // n of each system in btc
-    int nmax_btc = 0, nmax_bts = 0;
-    int *d_btc = nullptr, *d_bts = nullptr;
+    int nmax_btc = 0, nmax_bts = 0, nmax_btt = 0;
+    int *d_btc = nullptr, *d_bts = nullptr, *d_btt = nullptr;
     void* d_btjobs = nullptr;                          // 4 x count Tf3Job
     int nmax_rband = 0, nmax_rfull = 0;
     int nmax_all = 0, nmax_small = 0, nmax_large = 0, Mmax = 1, Dmax = 1;
@@ -643,12 +643,15 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
             b->sbt[bi].push_back(i);
             b->nmax_sbt[bi] = std::max(b->nmax_sbt[bi], (int)n);
         } else if (!d.small) {
-            (tc ? b->btc : b->bts).push_back(i);
+            // (systems the one-CTA reduction takes, unless a rule asks for the tensor cores)
+            const bool one = !tc && n < lmin && n <= mmf_hetrd_small_n(fp32);
+            (tc ? b->btc : one ? b->btt : b->bts).push_back(i);
             if (tc) {
                 b->btc_n.push_back((int)n);
                 b->nmax_btc = std::max(b->nmax_btc, (int)n);
             } else {
-                b->nmax_bts = std::max(b->nmax_bts, (int)n);
+                int& nm = one ? b->nmax_btt : b->nmax_bts;
+                nm = std::max(nm, (int)n);
             }
         }
         d.pan_off = b->n_pan;
@@ -695,7 +698,7 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
            o_status = p.take(sizeof(int) * count), o_rband = p.take(sizeof(int) * count),
            o_rfull = p.take(sizeof(int) * count), o_sbr = p.take(sizeof(int) * count), o_sbt = p.take(sizeof(int) * count),
            o_btc = p.take(sizeof(int) * count),
-           o_bts = p.take(sizeof(int) * count);
+           o_bts = p.take(sizeof(int) * count), o_btt = p.take(sizeof(int) * count);
     size_t o_coef = p.take(sizeof(double2) * b->n_coef);
     size_t o_H = p.take(cs * b->n_mat);
     size_t o_Zf = p.take(sizeof(double2) * b->n_mat);
@@ -767,6 +770,7 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
     b->d_rfull = (int*)(B + o_rfull);
     b->d_btc = (int*)(B + o_btc);
     b->d_bts = (int*)(B + o_bts);
+    b->d_btt = (int*)(B + o_btt);
     {  // the four window classes share one index array, one after another
         int* q = (int*)(B + o_sbr);
         for (int ci = 0; ci < 4; ++ci) {
@@ -855,6 +859,8 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
         if (e == cudaSuccess && !b->sbt[ci].empty())
             e = cudaMemcpyAsync(b->d_sbt[ci], b->sbt[ci].data(), sizeof(int) * b->sbt[ci].size(),
                                 cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !b->btt.empty())
+        e = cudaMemcpyAsync(b->d_btt, b->btt.data(), sizeof(int) * b->btt.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !b->bts.empty())
         e = cudaMemcpyAsync(b->d_bts, b->bts.data(), sizeof(int) * b->bts.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
@@ -866,7 +872,7 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
         return fail(MMF_ERR_CUDA, std::string("upload: ") + cudaGetErrorString(e));
     }
     // a side stream for each solver path of the reduction or the back-transform beyond the first
-    int nred = !b->medium.empty() + !b->tiny.empty(), nback = !b->bts.empty() + !b->btc.empty();
+    int nred = !b->medium.empty() + !b->tiny.empty(), nback = !b->bts.empty() + !b->btc.empty() + !b->btt.empty();
     for (int ci = 0; ci < 4; ++ci) nred += !b->sbr[ci].empty();
     for (int ci = 0; ci < 5; ++ci) nback += !b->sbt[ci].empty();
     const int nside = std::max(nred, nback) - 1;
@@ -1088,6 +1094,10 @@ static int launch_backtransforms(mmf_batch* b, Branches& br, int fp32) {
     if (!b->bts.empty()) {
         MmfLaunch Ls = on_stream(launch_of(b, b->bts, b->d_bts, b->nmax_bts), br.next());
         LAUNCH(mmf_launch_backtransform(Ls, b->d_H, b->d_tau, b->d_Vp, b->d_Y, b->d_Zp, fp32), 2);
+    }
+    if (!b->btt.empty()) {
+        MmfLaunch Lt = on_stream(launch_of(b, b->btt, b->d_btt, b->nmax_btt), br.next());
+        LAUNCH(mmf_launch_bt_small(Lt, b->d_H, b->d_tau, b->d_Y, b->d_Zp, fp32), 1);
     }
     return MMF_OK;
 }

@@ -268,6 +268,7 @@ int mmf_hetrd_max_n(int fp32);
 // mmf_hetrd_small_n
 int mmf_hetrd_small_n(int fp32);
 cudaError_t mmf_launch_hetrd_small(const MmfLaunch& L, void* H, double* dvec, double* evec, void* tau, int fp32);
+cudaError_t mmf_launch_bt_small(const MmfLaunch& L, const void* H, const void* tau, const double* Y, void* Z, int fp32);
 // banded H_F (k_sbr.cu): bulge chase to real tridiagonal form (d, e; reflectors kept in the
 // system's FP64 eigenvector slot), then Z = Q Y into the back-transform's output (Zp)
 int mmf_sbr_class(int band);                 // window class 8/16/32/64, 0 if the band is wider

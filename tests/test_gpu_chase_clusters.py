@@ -1,7 +1,8 @@
 """The band chase (k_sbr_chase) over its cluster sizes: one system takes the most CTAs its pipeline
 can use (8 from these sizes on), larger batches 4, 2 and 1 per system; bands at both ends of every
 window class, and dimensions one past a multiple of the band.  Quasienergies against LAPACK on the
-assembled matrix, to the library's bounds of 1e-12 ||H_F|| (FP64) and 1e-9 ||H_F|| (mixed)."""
+assembled matrix, to the library's bounds of 1e-12 ||H_F|| (FP64) and 1e-9 ||H_F|| (mixed); the
+eigenvectors (back-transform) by their residual and orthogonality."""
 
 import numpy as np
 import pytest
@@ -12,6 +13,7 @@ from paper_2005_03426_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 TOL = {M.MMF_FP64: 1e-12, M.MMF_MIXED: 1e-9}
+VEC = {M.MMF_FP64: 1e-10, M.MMF_MIXED: 1e-8}  # the library's bounds on U, which the eigenvectors carry
 
 
 def _check(problems, precision, at):
@@ -24,9 +26,14 @@ def _check(problems, precision, at):
     for i in at:
         assert b.path(i)[0] == M.MMF_PATH_BAND
         systems[i].build(M.MMF_FP64)
-        ref = np.linalg.eigvalsh(systems[i].hamiltonian())
-        E = b.get(i)[0]
-        assert np.abs(E - ref).max() <= TOL[precision] * np.abs(ref).max(), i
+        H = systems[i].hamiltonian()
+        ref = np.linalg.eigvalsh(H)
+        nrm = np.abs(ref).max()
+        E, Z = b.get(i)[0], b.eigenvectors(i)
+        assert np.abs(E - ref).max() <= TOL[precision] * nrm, i
+        # eigenvectors (the band back-transforms)
+        assert np.abs(H @ Z - Z * E[None, :]).max() <= VEC[precision] * nrm, i
+        assert np.abs(Z.conj().T @ Z - np.eye(systems[i].n)).max() <= VEC[precision], i
 
 
 # one mode, dense coupling: half-bandwidth 2 D - 1, n = D (2 N + 1)

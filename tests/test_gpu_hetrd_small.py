@@ -1,7 +1,8 @@
 """The one-CTA dense reduction (k_hetrd_small): dimensions at the edges of its 32-row groups and of its
 range (n up to 103 in FP64, 152 in FP32, the next size taking the cluster kernel), a system alone and
 in a batch of uneven ones.  Quasienergies against LAPACK on the assembled matrix, to the library's
-bounds of 1e-12 ||H_F|| (FP64) and 1e-9 ||H_F|| (mixed)."""
+bounds of 1e-12 ||H_F|| (FP64) and 1e-9 ||H_F|| (mixed); the back-transformed eigenvectors by their
+residual and orthogonality."""
 
 import numpy as np
 import pytest
@@ -12,6 +13,7 @@ from paper_2005_03426_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 TOL = {M.MMF_FP64: 1e-12, M.MMF_MIXED: 1e-9}
+VEC = {M.MMF_FP64: 1e-10, M.MMF_MIXED: 1e-8}  # the library's bounds on U, which the eigenvectors carry
 
 
 @pytest.mark.parametrize("precision", [M.MMF_FP64, M.MMF_MIXED])
@@ -29,5 +31,11 @@ def test_matches_lapack(precision, shapes):
     for i, s in enumerate(systems):
         assert b.path(i)[0] == M.MMF_PATH_DENSE
         s.build(M.MMF_FP64)
-        ref = np.linalg.eigvalsh(s.hamiltonian())
-        assert np.abs(b.get(i)[0] - ref).max() <= TOL[precision] * np.abs(ref).max(), i
+        H = s.hamiltonian()
+        ref = np.linalg.eigvalsh(H)
+        nrm = np.abs(ref).max()
+        E, Z = b.get(i)[0], b.eigenvectors(i)
+        assert np.abs(E - ref).max() <= TOL[precision] * nrm, i
+        # eigenvectors (the back-transform, k_bt_small)
+        assert np.abs(H @ Z - Z * E[None, :]).max() <= VEC[precision] * nrm, i
+        assert np.abs(Z.conj().T @ Z - np.eye(s.n)).max() <= VEC[precision], i
