@@ -145,8 +145,8 @@ template <> struct HtAcc<float2> {
 template <> struct HtAcc<double2> {
     double2 p;
     __device__ __forceinline__ HtAcc() : p(make_double2(0.0, 0.0)) {}
-    __device__ __forceinline__ void add(double2 a, double2 v, double2) { p = p + a * v; }
-    __device__ __forceinline__ void addc(double2 a, double2 v, double2) { p = p + cmulc(a, v); }
+    __device__ __forceinline__ void add(double2 a, double2 v, double2) { p = cmac(p, a, v); }
+    __device__ __forceinline__ void addc(double2 a, double2 v, double2) { p = cmacc(p, a, v); }
     __device__ __forceinline__ double2 mul() const { return p; }
     __device__ __forceinline__ double2 mulc() const { return p; }
 };
@@ -538,8 +538,8 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                     const C x0 = CG == 1 ? col[r] : acc;
 #pragma unroll 8
                     for (int c = grp; c < i; c += CG) {
-                        acc = acc + V[r + (int64_t)c * ld] * wk[c];
-                        acc2 = acc2 + W[r + (int64_t)c * ld] * vk[c];
+                        acc = cmac(acc, V[r + (int64_t)c * ld], wk[c]);
+                        acc2 = cmac(acc2, W[r + (int64_t)c * ld], vk[c]);
                     }
                     if (CG == 1) finish(r, x0, acc + acc2);
                 }
@@ -618,10 +618,10 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                     const int r = (q0 + CL * t) * 32 + lane;
                     if (r > k && r < n) {
                         const C v = vS[r - k - 1];
-                        s0 = s0 + cmulc(Wa[r], v);
-                        s1 = s1 + cmulc(Va[r], v);
-                        s2 = s2 + cmulc(Wb[r], v);
-                        s3 = s3 + cmulc(Vb[r], v);
+                        s0 = cmacc(s0, Wa[r], v);
+                        s1 = cmacc(s1, Va[r], v);
+                        s2 = cmacc(s2, Wb[r], v);
+                        s3 = cmacc(s3, Vb[r], v);
                     }
                 }
 #pragma unroll
@@ -680,8 +680,8 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                 if (r > k && r < n) {
 #pragma unroll 8
                     for (int c = grp; c < i; c += CG) {
-                        acc = acc + V[r + (int64_t)c * ld] * wk[c];
-                        acc2 = acc2 + W[r + (int64_t)c * ld] * vk[c];
+                        acc = cmac(acc, V[r + (int64_t)c * ld], wk[c]);
+                        acc2 = cmac(acc2, W[r + (int64_t)c * ld], vk[c]);
                     }
                     if (CG == 1) form_w(r - k - 1, acc + acc2);
                 }
@@ -780,7 +780,7 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
 #pragma unroll
                             for (int q = 0; q < 8; ++q) {
                                 const int cc = cg + 8 * q;
-                                acc[q] = acc[q] + a * tWc[p * HT_TILE + cc] + b * tVc[p * HT_TILE + cc];
+                                acc[q] = cmac(cmac(acc[q], a, tWc[p * HT_TILE + cc]), b, tVc[p * HT_TILE + cc]);
                             }
                         }
                     }

@@ -12,7 +12,7 @@
 // warp-wide FP64 instruction per 64 cycles and scheduler, 19 cycles over the SM's four): the O(m^2)
 // steps run on all warps (the update over the packed triangle's entries in line, so that no lane idles
 // at a column's end), the O(m) ones a row per thread, and the scalars in one warp.  Measured in FP64
-// at n = 82: one system 1.23 ms (k_hetrd 4.3), 200 systems 2.06 ms (k_hetrd 8.4).
+// at n = 82: one system 1.0 ms (k_hetrd 4.3), 200 systems 1.5 ms (k_hetrd 8.4).
 #include "mmf_internal.h"
 
 #define HS_THREADS 512
@@ -92,10 +92,10 @@ k_hetrd_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, ty
                 };
                 int c = p;
                 for (; c + np < m; c += 2 * np) {  // two independent chains
-                    a0 = a0 + entry(c) * v[c];
-                    a1 = a1 + entry(c + np) * v[c + np];
+                    a0 = cmac(a0, entry(c), v[c]);
+                    a1 = cmac(a1, entry(c + np), v[c + np]);
                 }
-                if (c < m) a0 = a0 + entry(c) * v[c];
+                if (c < m) a0 = cmac(a0, entry(c), v[c]);
                 part[p * n + i] = a0 + a1;
             }
         }
@@ -134,7 +134,7 @@ k_hetrd_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, ty
             if (q * (q + 1) / 2 > uu) --q;
             const int c = m - 1 - q, i = m - 1 - (uu - q * (q + 1) / 2);
             // v_i conj(w_c) + w_i conj(v_c)
-            tri[e] = tri[e] - cmulc(w[c], v[i]) - cmulc(v[c], w[i]);
+            tri[e] = cmsubc(cmsubc(tri[e], w[c], v[i]), v[c], w[i]);
         }
         __syncthreads();
     }
@@ -145,8 +145,8 @@ k_hetrd_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, ty
 // Z in shared memory and applies the reflectors one by one, last first, each column's rows dealt over
 // HS_BT_RG threads.  FP64-bound like the reduction (8 n^3 / 2 real flops a system), with two barriers a
 // reflector, where the blocked form's T factors and 64-row tiles cost more than they save at these
-// sizes: n = 82 in FP64, one system 0.27 ms (k_larft and k_backtransform 1.27), 200 systems
-// 1.8 ms (4.65).
+// sizes: n = 82 in FP64, one system 0.27 ms (k_larft and k_backtransform 1.27), 200 systems 1.2 ms
+// (4.65).
 #define HS_BT_NC 16
 #define HS_BT_THREADS 128
 #define HS_BT_RG (HS_BT_THREADS / HS_BT_NC)
@@ -189,10 +189,10 @@ k_bt_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, const
         C w = czero<C>(), w1 = w;
         int i = g;
         for (; i + HS_BT_RG < m; i += 2 * HS_BT_RG) {
-            w = w + cmulc(v[i], z[k + 1 + i][cl]);
-            w1 = w1 + cmulc(v[i + HS_BT_RG], z[k + 1 + i + HS_BT_RG][cl]);
+            w = cmacc(w, v[i], z[k + 1 + i][cl]);
+            w1 = cmacc(w1, v[i + HS_BT_RG], z[k + 1 + i + HS_BT_RG][cl]);
         }
-        if (i < m) w = w + cmulc(v[i], z[k + 1 + i][cl]);
+        if (i < m) w = cmacc(w, v[i], z[k + 1 + i][cl]);
         w = w + w1;
 #pragma unroll
         for (int o = HS_BT_NC; o < 32; o <<= 1) {
@@ -205,7 +205,7 @@ k_bt_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, const
 #pragma unroll
         for (int q = 1; q < HS_BT_THREADS / 32; ++q) w = w + red[q][cl];
         const C tw = t * w;
-        for (int q = g; q < m; q += HS_BT_RG) z[k + 1 + q][cl] = z[k + 1 + q][cl] - tw * v[q];
+        for (int q = g; q < m; q += HS_BT_RG) z[k + 1 + q][cl] = cmsub(z[k + 1 + q][cl], tw, v[q]);
         if (k > 0) {
             C* vn = vs[buf ^ 1];
             if (tx == 0) vn[0] = mk(R(1), R(0));

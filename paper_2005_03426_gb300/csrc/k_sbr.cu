@@ -75,8 +75,8 @@ template <> struct SbrAcc<float2> {
 template <> struct SbrAcc<double2> {
     double2 p;
     __device__ __forceinline__ SbrAcc() : p(make_double2(0.0, 0.0)) {}
-    __device__ __forceinline__ void add(double2 a, double2 v) { p = p + a * v; }
-    __device__ __forceinline__ void addc(double2 a, double2 v) { p = p + cmulc(v, a); }
+    __device__ __forceinline__ void add(double2 a, double2 v) { p = cmac(p, a, v); }
+    __device__ __forceinline__ void addc(double2 a, double2 v) { p = cmacc(p, v, a); }
     __device__ __forceinline__ double2 mul() const { return p; }
     __device__ __forceinline__ double2 mulc() const { return p; }
 };
@@ -85,12 +85,12 @@ __device__ __forceinline__ float2 sbr_sub_conj(float2 a, float2 f, float4 v) {
     a = __ffma2_rn(make_float2(-f.x, -f.y), make_float2(v.x, v.y), a);
     return __ffma2_rn(make_float2(-f.y, f.x), make_float2(v.z, v.w), a);
 }
-__device__ __forceinline__ double2 sbr_sub_conj(double2 a, double2 f, double2 v) { return a - cmulc(v, f); }
+__device__ __forceinline__ double2 sbr_sub_conj(double2 a, double2 f, double2 v) { return cmsubc(a, v, f); }
 __device__ __forceinline__ float2 sbr_sub(float2 a, float2 f, float4 v) {
     a = __ffma2_rn(make_float2(-f.x, -f.y), make_float2(v.x, v.y), a);
     return __ffma2_rn(make_float2(f.y, -f.x), make_float2(v.z, v.w), a);
 }
-__device__ __forceinline__ double2 sbr_sub(double2 a, double2 f, double2 v) { return a - f * v; }
+__device__ __forceinline__ double2 sbr_sub(double2 a, double2 f, double2 v) { return cmsub(a, f, v); }
 
 // Shared memory of one group.  B and D: the step's two blocks, column-major with a padded column
 // (LD even: two rows of a column are one aligned 16-byte read, and consecutive columns fall in
@@ -208,11 +208,11 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
 //
 // What bounds it: the critical path of about 2n steps of one sweep after another (a sweep starts two
 // steps behind its predecessor), so the latency of a step; on the FP64 path the 2 FP64 FMAs per clock
-// of an SM (about 25 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
+// of an SM (24 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
 // CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
 // b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
-// kernel): one system in FP32 36.2 -> 15.5 ms, 64 systems 37.4 -> 24.3 ms; eight systems in FP64
-// 455 -> 147 ms.
+// kernel): one system in FP32 36.2 -> 15.1 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
+// 455 -> 99 ms.
 //
 // CL = 1: one CTA per system.  CL > 1: a cluster of CL CTAs per system, the sweeps dealt round-robin
 // over all groups; a group reads its predecessor's progress key from that CTA's shared memory
@@ -593,8 +593,7 @@ __global__ void __launch_bounds__(128) k_sbr_bt_f32(const MmfDesc* __restrict__ 
 // FP64 instruction takes 64 cycles on its scheduler, 19 over the four): 8 n^3 flops per system at
 // least, which 8 systems of n = 1323 spread over the whole GPU do in 120 ms.  One column per thread
 // (128 columns per CTA) left 64 of 152 SMs idle there and took 417 ms; slabs of 32 and 16 columns keep
-// all four schedulers of a CTA's SM busy and spread evenly: 328 ms.  Rows past the band's b are
-// skipped.
+// all four schedulers of a CTA's SM busy and spread evenly: 213 ms.  Rows past the band's b are skipped.
 template <int BMAX, int NC>
 __global__ void __launch_bounds__(128) k_sbr_bt_f64(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                                                    const double2* __restrict__ store_base,
@@ -640,7 +639,7 @@ __global__ void __launch_bounds__(128) k_sbr_bt_f64(const MmfDesc* __restrict__ 
             for (int q = g; q < b; q += RG) {
                 int sl = top + q;
                 sl -= sl >= b ? b : 0;
-                w = w + cmulc(vs[buf][q], win[sl][cl]);
+                w = cmacc(w, vs[buf][q], win[sl][cl]);
             }
 #pragma unroll
             for (int o = NC; o < 32; o <<= 1) {
@@ -657,7 +656,7 @@ __global__ void __launch_bounds__(128) k_sbr_bt_f64(const MmfDesc* __restrict__ 
             for (int q = g; q < b; q += RG) {
                 int sl = top + q;
                 sl -= sl >= b ? b : 0;
-                const double2 z = win[sl][cl] - tw * vs[buf][q];
+                const double2 z = cmsub(win[sl][cl], tw, vs[buf][q]);
                 if (j > 0 && q == b - 1) {
                     if (act && r + q < n) Z[(int64_t)(r + q) * n + c] = z;
                 } else {

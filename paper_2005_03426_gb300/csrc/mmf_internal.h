@@ -73,6 +73,20 @@ template <> __device__ __forceinline__ float2 czero<float2>() { return make_floa
 MMF_CX_OPS(double2, double)
 MMF_CX_OPS(float2, float)
 
+// acc + a b, acc + conj(a) b, acc - a b and acc - conj(a) b as chains of four FMAs (written as a sum
+// of products the compiler takes six operations: multiply, FMA and add per component)
+#define MMF_CX_FMA(C)                                                                                       \
+    __device__ __forceinline__ C cmac(C s, C a, C b) {                                                      \
+        return mk(fma(-a.y, b.y, fma(a.x, b.x, s.x)), fma(a.y, b.x, fma(a.x, b.y, s.y)));                   \
+    }                                                                                                       \
+    __device__ __forceinline__ C cmacc(C s, C a, C b) {                                                     \
+        return mk(fma(a.y, b.y, fma(a.x, b.x, s.x)), fma(-a.y, b.x, fma(a.x, b.y, s.y)));                   \
+    }                                                                                                       \
+    __device__ __forceinline__ C cmsub(C s, C a, C b) { return cmac(s, mk(-a.x, -a.y), b); }                \
+    __device__ __forceinline__ C cmsubc(C s, C a, C b) { return cmacc(s, mk(-a.x, -a.y), b); }
+MMF_CX_FMA(double2)
+MMF_CX_FMA(float2)
+
 __device__ __forceinline__ double2 to_c128(double2 a) { return a; }
 __device__ __forceinline__ double2 to_c128(float2 a) { return make_double2(a.x, a.y); }
 template <class C> __device__ __forceinline__ C from_c128(double2 a);
