@@ -117,11 +117,6 @@ template <> struct TriP<float> {
 };
 
 // Power of two 2^-e with e the exponent of v (v > 0 finite), so that v 2^-e lies in [0.5, 1).
-__device__ __forceinline__ double pow2_below(double v) {
-    int ex;
-    frexp(v, &ex);
-    return ldexp(1.0, -ex);
-}
 __device__ __forceinline__ float pow2_below(float v) {
     // exponent field of a normal float; subnormal or zero v takes the scale 2^126
     const int be = (__float_as_int(v) >> 23) & 0xff;
@@ -137,53 +132,57 @@ __device__ __forceinline__ float pow2_below(float v) {
 // pair (p_i, p_{i-1}) is rescaled by the power of two that brings the larger of the two below
 // 1, which changes no sign; with ||T|| <= 1 (FP32) a step grows the pair by at most 3, and in
 // FP64 the exponent range leaves room for 16 steps at any ||T|| the workloads produce.
-// de2[i] = (d_i, e_{i-1}^2) with e_{-1} = 0.
-template <class R, class R2>
-__device__ __forceinline__ int sturm_count(const R2* __restrict__ de2, int n, R x) {
-    int cnt = 0;
-    R pm = R(1), p = de2[0].x - x;
-    if (p == R(0)) p = -TriP<R>::tiny();
-    cnt += (p < R(0));
-    for (int i = 1; i < n; ++i) {
-        const R2 v = de2[i];
-        R pn = fma(v.x - x, p, -v.y * pm);
-        if (pn == R(0)) pn = (p < R(0)) ? TriP<R>::tiny() : -TriP<R>::tiny();
-        cnt += ((pn < R(0)) != (p < R(0)));
-        pm = p;
-        p = pn;
-        if ((i & TriP<R>::rescale_mask) == 0) {
-            const R sc = pow2_below(fmax(fabs(p), fabs(pm)));
-            p *= sc;
-            pm *= sc;
-        }
-    }
-    return cnt;
+// Signs, zeros and the scale are taken from the bits: an FP64 comparison costs a warp the 64 cycles of
+// an FP64 operation, of which a step then has three (it had six).  A block's entries are loaded ahead
+// of its steps, which form one dependent chain.
+__device__ __forceinline__ uint32_t tri_hi(double v) { return (uint32_t)__double2hiint(v); }
+__device__ __forceinline__ uint32_t tri_hi(float v) { return (uint32_t)__float_as_int(v); }
+__device__ __forceinline__ bool tri_zero(double v) {
+    return ((tri_hi(v) << 1) | (uint32_t)__double2loint(v)) == 0u;
 }
+__device__ __forceinline__ bool tri_zero(float v) { return (tri_hi(v) << 1) == 0u; }
+// 2^-e with e the exponent of the larger of |p| and |q| (that one times 2^-e lies in [0.5, 1))
+__device__ __forceinline__ double tri_scale(double p, double q) {
+    const uint32_t a = tri_hi(p) & 0x7ff00000u, b = tri_hi(q) & 0x7ff00000u;
+    const int f = 2045 - (int)((a > b ? a : b) >> 20);
+    return __hiloint2double((f < 1 ? 1 : f > 2046 ? 2046 : f) << 20, 0);
+}
+__device__ __forceinline__ float tri_scale(float p, float q) { return pow2_below(fmaxf(fabsf(p), fabsf(q))); }
 
-// FP64 solver input: d and e^2 read from their own arrays.
-struct De2View {
-    const double* d;
-    const double* e2;
-    __device__ __forceinline__ double2 operator[](int i) const {
-        return make_double2(d[i], i > 0 ? e2[i - 1] : 0.0);
-    }
-};
-__device__ __forceinline__ int sturm_count(const De2View& v, int n, double x) {
-    int cnt = 0;
-    double pm = 1.0, p = v.d[0] - x;
-    if (p == 0.0) p = -1e-300;
-    cnt += (p < 0.0);
-    for (int i = 1; i < n; ++i) {
-        double pn = fma(v.d[i] - x, p, -v.e2[i - 1] * pm);
-        if (pn == 0.0) pn = (p < 0.0) ? 1e-300 : -1e-300;
-        cnt += ((pn < 0.0) != (p < 0.0));
+template <class R, class In>
+__device__ __forceinline__ int sturm_count(const In& in, int n, R x) {
+    constexpr int B = TriP<R>::rescale_mask + 1;  // steps between rescalings
+    R pm = R(1), p = in.dv(0) - x;
+    if (tri_zero(p)) p = -TriP<R>::tiny();
+    uint32_t hp = tri_hi(p);
+    int cnt = (int)(hp >> 31);
+    auto step = [&](R dv, R e2) {
+        R pn = fma(dv - x, p, -e2 * pm);
+        uint32_t hn = tri_hi(pn);
+        if (tri_zero(pn)) {
+            pn = (hp >> 31) ? TriP<R>::tiny() : -TriP<R>::tiny();
+            hn = tri_hi(pn);
+        }
+        cnt += (int)((hn ^ hp) >> 31);
         pm = p;
         p = pn;
-        if ((i & 15) == 0) {
-            const double sc = pow2_below(fmax(fabs(p), fabs(pm)));
-            p *= sc;
-            pm *= sc;
-        }
+        hp = hn;
+    };
+    int i = 1;
+    for (; i + B <= n; i += B) {
+        R dv[B], e2[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) in.de2(i + u, dv[u], e2[u]);
+#pragma unroll
+        for (int u = 0; u < B; ++u) step(dv[u], e2[u]);
+        const R sc = tri_scale(p, pm);
+        p *= sc;
+        pm *= sc;
+    }
+    for (; i < n; ++i) {
+        R dv, e2;
+        in.de2(i, dv, e2);
+        step(dv, e2);
     }
     return cnt;
 }
@@ -193,34 +192,47 @@ template <class R> struct TriIn;
 template <> struct TriIn<double> {
     const double* d;
     const double* e;
-    De2View de2;
+    const double* e2;
     double scale;
     __device__ TriIn(const MmfDesc& ds, const double* dvec, const double* evec, const double* e2vec,
                      const double*, const float*) {
         d = dvec + ds.vec_off;
         e = evec + ds.vec_off;
-        de2.d = d;
-        de2.e2 = e2vec + ds.vec_off;
+        e2 = e2vec + ds.vec_off;
         scale = 1.0;
     }
     __device__ __forceinline__ double dv(int i) const { return d[i]; }
     __device__ __forceinline__ double ev(int i) const { return e[i]; }
+    // d_i and e_{i-1}^2 (i >= 1)
+    __device__ __forceinline__ void de2(int i, double& a, double& b) const {
+        a = d[i];
+        b = e2[i - 1];
+    }
 };
 template <> struct TriIn<float> {
-    const float2* de2;
+    const float2* pairs;  // (d_i, e_{i-1}^2)
     const float* e;
     double scale;
     __device__ TriIn(const MmfDesc& ds, const double*, const double*, const double*, const double* aux_sys,
                      const float* fwork) {
         const int n = ds.n;
-        de2 = tri_f32_de2(fwork, ds);
-        e = (const float*)(de2 + n);
+        pairs = tri_f32_de2(fwork, ds);
+        e = (const float*)(pairs + n);
         scale = aux_sys[4];
     }
-    __device__ __forceinline__ float dv(int i) const { return de2[i].x; }
+    __device__ __forceinline__ float dv(int i) const { return pairs[i].x; }
     __device__ __forceinline__ float ev(int i) const { return e[i]; }
+    __device__ __forceinline__ void de2(int i, float& a, float& b) const {
+        const float2 v = pairs[i];
+        a = v.x;
+        b = v.y;
+    }
 };
 
+// L lanes per eigenvalue (a power of two up to 32): each iteration counts at L points that cut the
+// bracket into L + 1 parts, so a bracket takes log2(L + 1) bits a pass.  A pass is one dependent chain of
+// n steps; with few eigenvalues the schedulers that would idle take the other points (one system of
+// n = 82 in FP64 1160 -> BIS_ONE us, of n = 1323 in FP32 1560 -> BIS_F32 us).
 template <class R>
 __global__ void __launch_bounds__(128) k_bisect(const MmfDesc* __restrict__ descs,
                                                 const int* __restrict__ idx,
@@ -229,12 +241,13 @@ __global__ void __launch_bounds__(128) k_bisect(const MmfDesc* __restrict__ desc
                                                 const double* __restrict__ aux,
                                                 const float* __restrict__ fwork,
                                                 double* __restrict__ Eout,
-                                                int* __restrict__ status) {
+                                                int* __restrict__ status, int L) {
     const int sid = idx[blockIdx.y];
     const MmfDesc d = descs[sid];
     const int n = d.n;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) / L;
+    if ((int)(blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / L >= n) return;  // whole warps
+    const bool own = k < n;  // the warp's last lanes may lie past the last eigenvalue
     const TriIn<R> in(d, dvec, dvec, e2vec, aux + 8 * sid, fwork);
     const double sc = in.scale;
     // bracket and tolerances in the working precision (scaled for FP32; rounded outwards)
@@ -252,16 +265,32 @@ __global__ void __launch_bounds__(128) k_bisect(const MmfDesc* __restrict__ desc
     }
     const R eps = TriP<R>::eps();
     int it = 0;
+    const int lane = threadIdx.x & 31, g0 = lane & ~(L - 1), jl = lane - g0;  // first lane of the group, own place
+    const uint32_t gmask = L == 32 ? 0xffffffffu : ((1u << L) - 1u) << g0;
+    bool done = !own;
     for (; it < 200; ++it) {
-        R tol = fmax(R(2) * eps * fmax(fabs(lo), fabs(hi)), eps * tn) + pivmin;
-        if (hi - lo <= tol) break;
-        R mid = R(0.5) * (lo + hi);
-        if (mid <= lo || mid >= hi) break;
-        if (sturm_count(in.de2, n, mid) <= k) lo = mid;
-        else hi = mid;
+        if (!done) {
+            const R tol = fmax(R(2) * eps * fmax(fabs(lo), fabs(hi)), eps * tn) + pivmin;
+            const R mid = R(0.5) * (lo + hi);
+            done = hi - lo <= tol || mid <= lo || mid >= hi;
+        }
+        if (__all_sync(0xffffffffu, done)) break;
+        // this lane's point (a point that rounds onto an end of the bracket counts as that end does)
+        const R x = L == 1 ? R(0.5) * (lo + hi) : lo + (hi - lo) * (R(jl + 1) / R(L + 1));
+        const bool below = !done && (x <= lo || (x < hi && sturm_count<R>(in, n, x) <= k));
+        // the points up to the first one that is not below eigenvalue k raise lo, that one lowers hi
+        const uint32_t fails = ~__ballot_sync(0xffffffffu, below) & gmask;
+        const int first = fails ? __ffs(fails) - 1 : g0 + L;
+        const R xl = __shfl_sync(0xffffffffu, x, first > g0 ? first - 1 : g0);
+        const R xh = __shfl_sync(0xffffffffu, x, first < g0 + L ? first : g0);
+        if (!done) {
+            if (first > g0 && xl > lo) lo = xl;
+            if (first < g0 + L && xh < hi) hi = xh;
+        }
     }
+    if (!own || jl != 0) return;
     Eout[d.vec_off + k] = (0.5 * ((double)lo + (double)hi)) / sc;
-    if (it >= 200) status[sid] = MMF_ST_NOCONV;
+    if (!done) status[sid] = MMF_ST_NOCONV;
 }
 
 // Quotient for the elimination: correctly rounded in FP64; in FP32 the fast reciprocal-based
@@ -599,13 +628,21 @@ cudaError_t mmf_launch_tridiag_eig(const MmfLaunch& L, const double* dvec, const
     if (L.count <= 0) return cudaSuccess;
     k_tri_prep<<<L.count, 256, 0, L.stream>>>(L.desc, L.idx, dvec, evec, aux, e2, fp32 ? (float*)work : nullptr);
     dim3 g((L.nmax + 127) / 128, L.count);
+    // lanes per eigenvalue: while they find a free scheduler (FP64, whose units a warp fills) or leave
+    // the chains' latency to hide behind one another (FP32: four warps a scheduler)
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int lanes = 1;
+    while (lanes < 32 && (int64_t)L.count * L.nmax * 2 * lanes <= (int64_t)sms * (fp32 ? 512 : 128)) lanes *= 2;
+    dim3 gs((unsigned)(((int64_t)L.nmax * lanes + 127) / 128), L.count);
     if (fp32) {
-        k_bisect<float><<<g, 128, 0, L.stream>>>(L.desc, L.idx, dvec, e2, aux, (const float*)work, E, status);
+        k_bisect<float><<<gs, 128, 0, L.stream>>>(L.desc, L.idx, dvec, e2, aux, (const float*)work, E, status, lanes);
         k_inviter<float><<<g, 128, 0, L.stream>>>(L.desc, L.idx, dvec, evec, aux, E, Y, work, iters);
         k_cluster_cgs2_f32<<<dim3(L.nmax, L.count), CL_THREADS, 0, L.stream>>>(L.desc, L.idx, aux, E, work);
         k_widen_y_f32<<<dim3(256, L.count), 256, 0, L.stream>>>(L.desc, L.idx, work, Y);
     } else {
-        k_bisect<double><<<g, 128, 0, L.stream>>>(L.desc, L.idx, dvec, e2, aux, nullptr, E, status);
+        k_bisect<double><<<gs, 128, 0, L.stream>>>(L.desc, L.idx, dvec, e2, aux, nullptr, E, status, lanes);
         k_inviter<double><<<g, 128, 0, L.stream>>>(L.desc, L.idx, dvec, evec, aux, E, Y, work, iters);
     }
     return cudaGetLastError();
