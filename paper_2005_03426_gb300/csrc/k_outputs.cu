@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256) k_transition_avg(const MmfDesc* __restric
                     double2 amp = make_double2(0.0, 0.0);
                     for (int l = lam; l < c1; ++l) {
                         const double2* zc = Z + (int64_t)l * d.ld;
-                        amp = amp + cmulc(zc[i + D * d.b0], zc[r]);
+                        amp = cmacc(amp, zc[i + D * d.b0], zc[r]);
                     }
                     atomicAdd(&Ps[i * D + j], abs2(amp));
                 }
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(256) k_pbar_clusters(const MmfDesc* __restrict
                 const double2* zb = Z + (int64_t)l2 * d.ld;
                 for (int j = threadIdx.x; j < D; j += blockDim.x) {
                     double2 acc = make_double2(0.0, 0.0);
-                    for (int b = 0; b < M; ++b) acc = acc + cmulc(zb[j + D * b], za[j + D * b]);
+                    for (int b = 0; b < M; ++b) acc = cmacc(acc, zb[j + D * b], za[j + D * b]);
                     Sj[j] = acc;  // sum_b Z[(j,b),l] conj(Z[(j,b),l2])
                 }
                 __syncthreads();

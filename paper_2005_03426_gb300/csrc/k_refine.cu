@@ -964,12 +964,12 @@ __global__ void __launch_bounds__(256) k_cluster_sep(const MmfDesc* __restrict__
                                 const int e2 = (mq + 1) * D + i;
                                 for (int k = 0; k < cnt[e2]; ++k) {
                                     const int j = jx[(int64_t)e2 * cap + k];
-                                    acc = acc + cmulc(V[j * D + i], xd[j]);
+                                    acc = cmacc(acc, V[j * D + i], xd[j]);
                                 }
                             } else {
                                 for (int j = 0; j < D; ++j) {
                                     const double2 v = V[j * D + i];
-                                    if (v.x != 0.0 || v.y != 0.0) acc = acc + cmulc(v, xd[j]);
+                                    if (v.x != 0.0 || v.y != 0.0) acc = cmacc(acc, v, xd[j]);
                                 }
                             }
                         }
@@ -987,8 +987,8 @@ __global__ void __launch_bounds__(256) k_cluster_sep(const MmfDesc* __restrict__
                 const double2* hq = HX + (int64_t)(c0 + q) * d.ld;
                 double2 acc = make_double2(0.0, 0.0), gac = make_double2(0.0, 0.0);
                 for (int r = threadIdx.x & 31; r < n; r += 32) {
-                    acc = acc + cmulc(xp[r], hq[r]);
-                    gac = gac + cmulc(xp[r], xq[r]);
+                    acc = cmacc(acc, xp[r], hq[r]);
+                    gac = cmacc(gac, xp[r], xq[r]);
                 }
                 acc.x = warp_sum(acc.x);
                 acc.y = warp_sum(acc.y);
