@@ -12,7 +12,7 @@
 // spread over the grid because they read the panel (m x 2i entries): one CTA streamed it at a few tens
 // of GB/s, as long as the gemv over the whole trailing matrix.  A column is bound by its launches until
 // m is several thousand (n = 5832: 48 us a column, of which the lower triangle's reads at the copy rate
-// take 13; with six launches and a row per thread 286 ms, with four and four threads a row 172), so there
+// take 13; with six launches and a row per thread 286 ms, with four and four threads a row 167), so there
 // are as few as the dependences allow, and each is launched with programmatic
 // stream serialisation: its CTAs are set up while the previous kernel drains and wait for it at their
 // start.  After each panel a grid-wide
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(256) k_lg_her2k(typename Cx<R>::T* __restrict_
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 const int cc = cg + 4 * q;
-                acc[q] = acc[q] + a * tWc[p][cc] + b * tVc[p][cc];
+                acc[q] = cmac(cmac(acc[q], a, tWc[p][cc]), b, tVc[p][cc]);
             }
         }
     }

@@ -42,7 +42,7 @@ int64_t mmf_sbr_store_elems(int n, int b) { return sbr_nref(n, b) * (b + 1); }
 #define SBR_WAIT_LIMIT (1 << 26)
 // bytes before the groups' blocks in dynamic shared memory (progress keys, abort flag), rounded to
 // 256 so that the blocks' 16-byte complex elements stay aligned
-__host__ __device__ constexpr int sbr_hdr(int ng) { return (8 * ng + 16 + 255) / 256 * 256; }
+__host__ __device__ constexpr int sbr_hdr(int ng) { return (16 * ng + 16 + 255) / 256 * 256; }
 
 // A vector entry in shared memory as the multiplier of packed products: (x, x), (y, y).  With it
 // acc1 += a (x, x) and acc2 += a (y, y) are two packed FP32 instructions, and
@@ -106,7 +106,8 @@ struct __align__(16) SbrGroup {
     C red[3][P][BMAX];   // partial sums: B v_p, v^H B, D v
     C c0[BMAX];          // B(:, 0)
     C ty[BMAX];
-    C beta[2];
+    C dl[BMAX];          // D's last row and B's last entry, taken from the predecessor's published row
+    C bl, beta, d00, pad;
 };
 
 // Predicated load (zero where !ok) and store of one complex element, without a branch around each.
@@ -204,15 +205,22 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
 // from its loads to its stores; a copy in shared memory serves the sums down the columns.  A step is
 //   load | y = B v_p (partial sums) | x = B(:,0) - tau_p y gives v, tau, beta | u = v^H B and D v
 //   (rows from registers, columns from shared memory) | w vectors | rank-2 updates, store
-// with five group barriers; one warp computes the vectors.
+// with five group barriers; one warp computes the vectors.  A successor's step s needs all but its last
+// row from the predecessor's step s, and that row (B's is zero but for its last entry, beta) from the
+// first row of the predecessor's step s + 1: one warp computes and publishes that row as soon as the
+// step's vectors are known, so a sweep follows its predecessor by a step and the part of a step up to
+// there, with its loads and B v_p done beforehand, where it waited for two whole steps (one FP32 system
+// of n = 1323 15.1 -> 13.2 ms, eight in FP64 99 -> 87).  With few groups per system (CL <= 2 and wide
+// windows) the SMs are busy anyway and the publication's fence costs 5 %: there a sweep waits for all of
+// the predecessor's step s + 1.
 //
-// What bounds it: the critical path of about 2n steps of one sweep after another (a sweep starts two
-// steps behind its predecessor), so the latency of a step; on the FP64 path the 2 FP64 FMAs per clock
+// What bounds it: the critical path of one sweep after another (about 1.5 n steps), so the latency of a
+// step; on the FP64 path the 2 FP64 FMAs per clock
 // of an SM (24 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
 // CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
 // b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
-// kernel): one system in FP32 36.2 -> 15.1 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
-// 455 -> 99 ms.
+// kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
+// 455 -> 87 ms.
 //
 // CL = 1: one CTA per system.  CL > 1: a cluster of CL CTAs per system, the sweeps dealt round-robin
 // over all groups; a group reads its predecessor's progress key from that CTA's shared memory
@@ -234,10 +242,12 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
     constexpr int SL = BMAX >= 32 ? BMAX / 32 : 1;  // entries of a vector per lane
     constexpr bool F64 = sizeof(R) == 8;            // FP64 units are scarce: skip padding
     constexpr int NGT = CL * NG;                    // groups per system
+    constexpr bool EARLY = CL >= 4 || NG >= 8;      // first rows published ahead
     static_assert(G % 32 == 0 && EL * P == BMAX && EL % 2 == 0, "group shape");
     extern __shared__ __align__(16) unsigned char sbr_smem[];
     long long* key = reinterpret_cast<long long*>(sbr_smem);
-    int* abort_flag = reinterpret_cast<int*>(sbr_smem + 8 * NG);
+    long long* pub = key + NG;
+    int* abort_flag = reinterpret_cast<int*>(sbr_smem + 16 * NG);
     Grp* groups = reinterpret_cast<Grp*>(sbr_smem + sbr_hdr(NG));
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = CL > 1 ? (int)cluster.block_rank() : 0;
@@ -259,10 +269,11 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
     const long long KK = sbr_passes(n, b) + 3;
     // the predecessor sweep's group, its progress key and its CTA's abort flag
     const int ggp = (gg + NGT - 1) % NGT;
-    const uint32_t pkey = map_rank(key + ggp % NG, ggp / NG), pabort = map_rank(abort_flag, ggp / NG);
-    const uint32_t mykey = map_rank(key + g, rank);
+    const uint32_t pkey = map_rank(key + ggp % NG, ggp / NG), ppub = map_rank(pub + ggp % NG, ggp / NG);
+    const uint32_t pabort = map_rank(abort_flag, ggp / NG);
+    const uint32_t mykey = map_rank(key + g, rank), mypub = map_rank(pub + g, rank);
 
-    if (threadIdx.x < NG) key[threadIdx.x] = -1;
+    if (threadIdx.x < 2 * NG) key[threadIdx.x] = -1;
     if (threadIdx.x == 0) *abort_flag = 0;
     if (CL > 1) cluster.sync(); else __syncthreads();
     if (threadIdx.x == 0 && rank == 0) dd[0] = (double)Hg[0].x;
@@ -275,51 +286,58 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
     int cur = 0;  // buffer of the current reflector in S.v
     bool stopped = false;
     C tau = zero, taup = zero;
+    // a warp's bounded wait for a predecessor's progress (acquire); after one gave up nobody waits
+    auto wait_for = [&](uint32_t where, long long need) {
+        if (stopped) return;
+        if (lane == 0) {
+            int it = 0;
+            while (key_load(where) < need) {
+                const int gave_up = ++it > SBR_WAIT_LIMIT;
+                if (gave_up || flag_load(pabort) || *(volatile int*)abort_flag) {
+                    *(volatile int*)abort_flag = 1;  // the successors' CTAs see it too
+                    status[sid] = MMF_ST_NOCONV;
+                    stopped = true;
+                    break;
+                }
+                __nanosleep(32);
+            }
+        }
+        stopped = __shfl_sync(0xffffffffu, stopped, 0);
+    };
     for (int j = gg; j <= n - 2; j += NGT) {
         const int nsteps = (n - 2 - j) / b + 1;
         for (int s = 0; s < nsteps; ++s) {
-            // wait until sweep j-1 has finished step s+1 (or all of its steps)
-            if (j > 0 && !stopped) {
-                if (lane == 0) {
-                    const long long need = (long long)(j - 1) * KK + (s + 2 < KK - 1 ? s + 2 : KK - 1);
-                    int it = 0;
-                    while (key_load(pkey) < need) {
-                        const int gave_up = ++it > SBR_WAIT_LIMIT;
-                        if (gave_up || flag_load(pabort) || *(volatile int*)abort_flag) {
-                            *(volatile int*)abort_flag = 1;  // the successors' CTAs see it too
-                            status[sid] = MMF_ST_NOCONV;
-                            stopped = true;
-                            break;
-                        }
-                        __nanosleep(32);
-                    }
-                }
-                stopped = __shfl_sync(0xffffffffu, stopped, 0);
-            }
+            // rows r .. r + b - 2 are the predecessor's of its step s, which it has to have finished;
+            // row r + b - 1, if there is one, is the first row of its step s + 1, published during it
+            // (without publication: all of step s + 1)
+            if (j > 0) wait_for(pkey, (long long)(j - 1) * KK + (EARLY ? s + 1 : s + 2 < KK - 1 ? s + 2 : KK - 1));
             const int r = j + 1 + s * b, rp = r - b;
             const int l = min(b, n - r);
+            const bool late = EARLY && j > 0 && l == b;
+            const int lim = late ? b - 1 : l;
             // (a) the step's entries: all loads in flight together, zeros outside the blocks
             C B[EL], D[EL], x[SL];
             {
                 const C* h = Hg + (r + k0) * ldi + r + i;
 #pragma unroll
                 for (int q = 0; q < EL; ++q)
-                    D[q] = ld_if<(CL > 1)>(h + q * ldi, i < l && i >= k0 + q);
+                    D[q] = ld_if<(CL > 1)>(h + q * ldi, i < lim && i >= k0 + q);
             }
             if (s > 0) {
                 const C* h = Hg + (rp + k0) * ldi + r + i;
 #pragma unroll
                 for (int q = 0; q < EL; ++q)
-                    B[q] = ld_if<(CL > 1)>(h + q * ldi, i < l && k0 + q < b);
+                    B[q] = ld_if<(CL > 1)>(h + q * ldi, i < lim && k0 + q < b);
             } else if (warp == 0) {
 #pragma unroll
                 for (int u = 0; u < SL; ++u) {
                     const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
-                    x[u] = ld_if<(CL > 1)>(Hg + j * ldi + r + e, e < l);
+                    x[u] = ld_if<(CL > 1)>(Hg + j * ldi + r + e, e < lim);
                 }
             }
 #pragma unroll
             for (int q = 0; q < EL; ++q) S.D[(k0 + q) * LD + i] = i == k0 + q ? zero : D[q];
+            if (tid == 0) S.d00 = D[0];
             if (s > 0) {
                 // y = B v_p over this thread's columns
                 const auto* vp = S.v[cur ^ 1] + k0;
@@ -344,6 +362,24 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             R beta = R(0);
             if (warp == 0) {
                 R part = R(0);
+                C bl = zero;  // B(b-1, b-1), the only nonzero of B's last row; at s = 0 x(b-1)
+                if (late) {
+                    wait_for(ppub, (long long)(j - 1) * KK + (s + 2));
+                    const C* h = Hg + r + b - 1;
+                    bl = ld_if<(CL > 1)>(h + (r - 1) * ldi, true);
+#pragma unroll
+                    for (int u = 0; u < SL; ++u) {
+                        const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                        const C dl = ld_if<(CL > 1)>(h + (r + (e < b ? e : 0)) * ldi, e < b);
+                        S.dl[e] = dl;
+                        if (e < b - 1) S.D[e * LD + b - 1] = dl;
+                        if (s == 0 && e == b - 1) x[u] = bl;
+                    }
+                    if (lane == 0) {
+                        S.bl = bl;
+                        if (s > 0) S.B[(b - 1) * LD + b - 1] = bl;
+                    }
+                }
                 if (s > 0) {
 #pragma unroll
                     for (int u = 0; u < SL; ++u) {
@@ -351,8 +387,13 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                         C y = S.red[0][0][e];
 #pragma unroll
                         for (int q = 1; q < P; ++q) y = y + S.red[0][q][e];
+                        C c0 = S.c0[e];
+                        if (late && e == b - 1) {
+                            y = y + bl * DupC::val(S.v[cur ^ 1][b - 1]);
+                            if (b == 1) c0 = bl;
+                        }
                         ty[u] = taup * y;
-                        x[u] = S.c0[e] - ty[u];   // v_p[0] = 1
+                        x[u] = c0 - ty[u];   // v_p[0] = 1
                         S.ty[e] = ty[u];
                     }
                 }
@@ -369,10 +410,17 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                     vl[u] = e == 0 ? mk(R(1), R(0)) : x[u] * scale;
                     S.v[cur][e] = DupC::of(vl[u]);
                 }
-                if (lane == 0) S.beta[0] = mk(beta, R(0));
+                if (lane == 0) S.beta = mk(beta, R(0));
             }
             gbar<G>(g);
             const auto* v = S.v[cur];
+            if (late && i == b - 1) {  // the owners of the last row
+#pragma unroll
+                for (int q = 0; q < EL; ++q) {
+                    if (k0 + q < b) D[q] = S.dl[k0 + q];
+                    if (s > 0 && k0 + q == b - 1) B[q] = S.bl;
+                }
+            }
             // (c) column i over rows k0 .. k0 + EL - 1 of B and of D's strict lower triangle, and row i
             // of D's lower triangle over columns k0 .. (warps whose share is zero skip it)
             {
@@ -439,8 +487,35 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                 }
             }
             gbar<G>(g);
-            // (e) rank-2 updates of this thread's entries, back to global memory
+            // the first row of both blocks, published at once for the successor, whose step s - 1 has it
+            // as its last row
+            if (EARLY && warp == G / 32 - 1) {
+                const auto* vp = S.v[cur ^ 1];
+#pragma unroll
+                for (int u = 0; u < SL; ++u) {
+                    const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
+                    C a = S.beta;
+                    if (s > 0 && e > 0)
+                        a = sbr_sub(sbr_sub_conj(S.B[e * LD], S.ty[0], vp[e]), mk(R(1), R(0)), S.wu[e]);
+                    st_if(Hg + (r - (s > 0 ? b - (e < b ? e : 0) : 1)) * ldi + r, a,
+                          (BMAX >= 32 || lane < BMAX) && e < b && (s > 0 || e == 0));
+                }
+                if (lane == 0) {
+                    const C w0 = DupC::val(S.wd[0]);
+                    C a = late && b == 1 ? S.dl[0] : S.d00;
+                    a = mk(a.x - R(2) * w0.x, R(0));  // v_0 = 1
+                    st_if(Hg + r * ldi + r, a, true);
+                    if (s == 0) {
+                        dd[j + 1] = (double)a.x;
+                        ee[j] = (double)S.beta.x;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) key_store(mypub, (long long)j * KK + (s + 1));
+            }
+            // (e) rank-2 updates of this thread's other entries, back to global memory
             const C vi = DupC::val(v[i]), wi = DupC::val(S.wd[i]);
+            const bool st = (!EARLY || i > 0) && i < l;
             if (s > 0) {
                 const C tyi = S.ty[i];
                 const auto *vp = S.v[cur ^ 1] + k0, *wu = S.wu + k0;
@@ -449,8 +524,8 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                 for (int q = 0; q < EL; ++q) {
                     if (F64 && k0 + q >= b) continue;
                     C a = sbr_sub(sbr_sub_conj(B[q], tyi, vp[q]), vi, wu[q]);
-                    if (q == 0 && p == 0) a = i == 0 ? S.beta[0] : zero;
-                    st_if(h + q * ldi, a, i < l && k0 + q < b);
+                    if (q == 0 && p == 0) a = i == 0 ? S.beta : zero;
+                    st_if(h + q * ldi, a, st && k0 + q < b);
                 }
             }
             if (row) {
@@ -463,8 +538,8 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                     // v_i conj(w_k) + w_i conj(v_k)
                     C a = sbr_sub_conj(sbr_sub_conj(D[q], vi, wd[q]), wi, vk[q]);
                     if (i == k) a.y = R(0);
-                    st_if(h + q * ldi, a, i >= k && i < l);
-                    if (q == 0 && s == 0 && tid == 0) dd[j + 1] = (double)a.x;
+                    st_if(h + q * ldi, a, st && i >= k);
+                    if (!EARLY && q == 0 && s == 0 && tid == 0) dd[j + 1] = (double)a.x;
                 }
             }
             if (warp == 0) {
@@ -472,9 +547,12 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
 #pragma unroll
                     for (int u = 0; u < SL; ++u) {
                         const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
-                        if (e < l) Hg[j * ldi + r + e] = e == 0 ? mk(beta, R(0)) : zero;
+                        if (e > 0 && e < l) Hg[j * ldi + r + e] = zero;
+                        if (!EARLY && e == 0 && lane == 0) {
+                            Hg[j * ldi + r] = mk(beta, R(0));
+                            ee[j] = (double)beta;
+                        }
                     }
-                    if (lane == 0) ee[j] = (double)beta;
                 }
                 // store the reflector for the back-transform, marked evict-first: the store is
                 // written once and read only after the chase, and L2 should keep the band's lines
@@ -744,7 +822,7 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
 // The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
 // pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
 // system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
-// take, with 8 it takes 15.5.
+// take, with 8 it takes 13.2.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
                                 int* status) {
