@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(256) k_pbar_clusters(const MmfDesc* __restrict
 // tensor-core path (mmf_launch_phi)
 cudaError_t mmf_launch_outputs(const MmfLaunch& L, int Mmax, int Dmax, const double* E,
                                   const double2* Z, float2* Z1, float2* Zlo, const double* t, double t0, int nt,
-                                  double2* F2, double2* U, double* P, double cluster_rel, int skip_u,
+                                  double2* F2, double2* U, double* P, double cluster_rel, int skip_u, int skip_p,
                                   void* scratch, int scratch_esz) {
     static_assert(sizeof(Split) == sizeof(double2), "phase table slots hold one Split each");
     Split* F = reinterpret_cast<Split*>(F2);
@@ -325,6 +325,7 @@ cudaError_t mmf_launch_outputs(const MmfLaunch& L, int Mmax, int Dmax, const dou
             k_time_evolution<<<dim3((L.nmax + 31) / 32, L.count), 256, 0, L.stream>>>(
                 L.desc, L.idx, E, Z, Z1, Zlo, t, t0, nt, F, U);
     }
+    if (skip_p) return cudaGetLastError();
     const int Ds = Dmax < PB_DSMALL ? Dmax : PB_DSMALL;
     size_t sm = sizeof(double) * (size_t)(Ds * Ds + 8 * Ds);
     if (sm > 48 * 1024) {

@@ -801,6 +801,34 @@ __global__ void __launch_bounds__(OZ_WARPS * 32, 1) k_oz_phi(const MmfDesc* __re
 #define PU_L 32
 #define PU_T 64
 #define PU_DMAX 16  // levels per system on this path (more take the double-FP32 kernel)
+// U's sums over one CTA's eigenvectors: thread (time, j) adds Phi_j(t, l) e^{-i E_l (t - t0)} conj(Z((i, b0), l))
+// over l for every i
+template <int DC>
+__device__ __forceinline__ void phi_u_sums(const double2* __restrict__ Phi, const double2 (*ph)[PU_T],
+                                           const double2 (*z0)[PU_DMAX], int D, int n, int l0, int nl, int tb, int ntt,
+                                           int nt, double2* __restrict__ Uo) {
+    const int nd = DC == PU_DMAX ? D : DC;
+    for (int task = threadIdx.x; task < ntt * D; task += blockDim.x) {
+        const int tt = task % ntt, j = task / ntt;
+        double2 acc[DC];
+#pragma unroll
+        for (int i = 0; i < DC; ++i) acc[i] = make_double2(0.0, 0.0);
+        for (int a = 0; a < nl; ++a) {
+            const double2 f = Phi[((int64_t)j * n + l0 + a) * nt + tb + tt] * ph[a][tt];
+#pragma unroll
+            for (int i = 0; i < DC; ++i)
+                if (DC < PU_DMAX || i < nd) acc[i] = cmacc(acc[i], z0[a][i], f);
+        }
+        double2* u = Uo + ((int64_t)(tb + tt) * D + j) * D;
+#pragma unroll
+        for (int i = 0; i < DC; ++i)
+            if (i < nd) {
+                atomicAdd(&u[i].x, acc[i].x);
+                atomicAdd(&u[i].y, acc[i].y);
+            }
+    }
+}
+
 __global__ void __launch_bounds__(256) k_phi_u(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
                                                const uint16_t* __restrict__ pool, const double* __restrict__ Eg,
                                                const double2* __restrict__ Zg, const double* __restrict__ tpool,
@@ -825,24 +853,19 @@ __global__ void __launch_bounds__(256) k_phi_u(const MmfDesc* __restrict__ descs
         z0[a][i] = a < nl ? Zg[d.mat_off + (int64_t)(l0 + a) * d.ld + i + D * d.b0] : make_double2(0.0, 0.0);
     }
     __syncthreads();
-    for (int task = threadIdx.x; task < ntt * D; task += blockDim.x) {
-        const int tt = task % ntt, j = task / ntt;
-        double2 acc[PU_DMAX];
-#pragma unroll
-        for (int i = 0; i < PU_DMAX; ++i) acc[i] = make_double2(0.0, 0.0);
-        for (int a = 0; a < nl; ++a) {
-            const double2 f = Phi[((int64_t)j * n + l0 + a) * nt + tb + tt] * ph[a][tt];
-#pragma unroll
-            for (int i = 0; i < PU_DMAX; ++i)
-                if (i < D) acc[i] = acc[i] + cmulc(z0[a][i], f);
-        }
-        double2* u = U + d.u_off + ((int64_t)(tb + tt) * D + j) * D;
-#pragma unroll
-        for (int i = 0; i < PU_DMAX; ++i)
-            if (i < D) {
-                atomicAdd(&u[i].x, acc[i].x);
-                atomicAdd(&u[i].y, acc[i].y);
-            }
+    double2* Uo = U + d.u_off;
+    // the level count as a constant up to 8 levels: the sums then are four chained FMAs each and nothing
+    // else (with a run-time bound the compiler issues all 16 levels' FP64 operations, switched off)
+    switch (D) {
+        case 1: phi_u_sums<1>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 2: phi_u_sums<2>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 3: phi_u_sums<3>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 4: phi_u_sums<4>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 5: phi_u_sums<5>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 6: phi_u_sums<6>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 7: phi_u_sums<7>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        case 8: phi_u_sums<8>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo); break;
+        default: phi_u_sums<PU_DMAX>(Phi, ph, z0, D, n, l0, nl, tb, ntt, nt, Uo);
     }
 }
 

@@ -150,6 +150,7 @@ struct mmf_batch {
     bool pinned = true;     // host staging buffers page-locked (false: pageable, for serving)
     bool times_set = false;
     int last_stage = 0;  // 1 assembled, 2 diagonalised, 3 outputs
+    bool p_valid = false;  // Pbar belongs to the present eigenpairs
     // per-stage CUDA-event timing (optional)
     int timing_runs = 0, runs_recorded = 0;
     std::vector<cudaEvent_t> ev;
@@ -1104,6 +1105,7 @@ static int launch_backtransforms(mmf_batch* b, Branches& br, int fp32) {
 
 static int stage_eig(mmf_batch* b) {
     const int fp32 = b->precision == MMF_MIXED;
+    b->p_valid = false;
     mark(b, ST_JACOBI);
     if (!b->small.empty()) {
         MmfLaunch Ls = launch_of(b, b->small, b->d_small, b->nmax_small);
@@ -1193,37 +1195,40 @@ static int stage_eig(mmf_batch* b) {
     return MMF_OK;
 }
 
-static int stage_outputs(mmf_batch* b) {
+// U and / or Pbar (a one-system call computes what it was asked for; a batch run both)
+static int stage_outputs(mmf_batch* b, bool want_u, bool want_p) {
     cudaStream_t st = b->stream;
     mark(b, ST_OUTPUTS);
-    if (b->n_u > 0) CU(cudaMemsetAsync(b->d_U, 0, sizeof(double2) * b->n_u, st));
-    CU(cudaMemsetAsync(b->d_P, 0, sizeof(double) * b->n_p, st));
+    const int nt = want_u ? b->nt : 0;
+    if (nt > 0) CU(cudaMemsetAsync(b->d_U, 0, sizeof(double2) * b->n_u, st));
+    if (want_p) CU(cudaMemsetAsync(b->d_P, 0, sizeof(double) * b->n_p, st));
     MmfLaunch La = launch_of(b, b->all, b->d_all, b->nmax_all);
     // FP32 pieces of Z: the mixed path reuses the refinement's X1 and T buffers (free by now)
     float2* Z1 = b->precision == MMF_MIXED ? b->d_X1 : b->d_Zs;
     float2* Zlo = b->precision == MMF_MIXED ? reinterpret_cast<float2*>(b->d_T) : b->d_Zs + b->n_mat;
     // mixed path: U on the tensor cores (exact slicing) unless a system has too many levels
     // (the int64 sums of the exact slicing bound K = 2M as they bound the Gram product's 2n)
-    const bool phi = b->precision == MMF_MIXED && b->nt > 0 && b->Dmax <= mmf_phi_max_levels() &&
+    const bool phi = b->precision == MMF_MIXED && nt > 0 && b->Dmax <= mmf_phi_max_levels() &&
                      b->Mmax <= mmf_ozaki_max_n();
-    LAUNCH(mmf_launch_outputs(La, b->Mmax, b->Dmax, b->d_E, b->d_Zf, Z1, Zlo, b->d_t, b->t0, b->nt, b->d_F,
-                              b->d_U, b->d_P, 1e-8, phi ? 1 : 0, b->d_H,
+    LAUNCH(mmf_launch_outputs(La, b->Mmax, b->Dmax, b->d_E, b->d_Zf, Z1, Zlo, b->d_t, b->t0, nt, b->d_F,
+                              b->d_U, b->d_P, 1e-8, phi ? 1 : 0, want_p ? 0 : 1, b->d_H,
                               b->precision == MMF_MIXED ? (int)sizeof(float2) : (int)sizeof(double2)),
-           b->nt > 0 ? (phi ? 3 : 4) : 1);
+           (nt > 0 ? (phi ? 2 : 3) : 0) + (want_p ? 1 : 0));
     if (phi)
-        LAUNCH(mmf_launch_phi(La, b->Dmax, b->nt, Z1, Zlo, b->d_F, b->d_E, b->d_Zf, b->d_t, b->t0, b->d_oz, b->d_U,
+        LAUNCH(mmf_launch_phi(La, b->Dmax, nt, Z1, Zlo, b->d_F, b->d_E, b->d_Zf, b->d_t, b->t0, b->d_oz, b->d_U,
                               b->d_status),
                4);
     mark(b, ST_COUNT);
     if (b->timing_runs > 0) b->runs_recorded++;
     b->last_stage = 3;
+    if (want_p) b->p_valid = true;
     return MMF_OK;
 }
 
 static int run_stages(mmf_batch* b) {
     int rc = stage_assemble(b);
     if (rc == MMF_OK) rc = stage_eig(b);
-    if (rc == MMF_OK) rc = stage_outputs(b);
+    if (rc == MMF_OK) rc = stage_outputs(b, true, true);
     return rc;
 }
 
@@ -1463,7 +1468,7 @@ static int solo_outputs(mmf_sys* s, double t0, int nt, const double* t) {
     }
     int rc = mmf_batch_set_times(b, t0, t);
     if (rc != MMF_OK) return rc;
-    return stage_outputs(b);
+    return stage_outputs(b, true, false);
 }
 
 extern "C" int mmf_time_evolution(mmf_sys* s, double t0, int nt, const double* t, double* U) {
@@ -1484,13 +1489,8 @@ extern "C" int mmf_transition_avg(mmf_sys* s, double* P) {
     std::lock_guard<std::recursive_mutex> lk(s->ctx->mu);
     CU(cudaSetDevice(s->ctx->device));
     mmf_batch* b = s->solo;
-    if (b->last_stage < 3) {
-        if (b->nt > 0 && !b->times_set) {
-            std::vector<double> z((size_t)b->nt, 0.0);
-            int rc = mmf_batch_set_times(b, 0.0, z.data());
-            if (rc != MMF_OK) return rc;
-        }
-        int rc = stage_outputs(b);
+    if (!b->p_valid) {
+        int rc = stage_outputs(b, false, true);
         if (rc != MMF_OK) return rc;
     }
     return mmf_batch_get(b, 0, nullptr, nullptr, P);
@@ -1604,7 +1604,7 @@ extern "C" int mmf_time_evolution_dev(mmf_sys* s, double t0, int nt, const doubl
     CU(cudaMemcpyAsync(b->d_t, t, sizeof(double) * nt, cudaMemcpyDeviceToDevice, b->stream));
     b->t0 = t0;
     b->times_set = true;
-    rc = stage_outputs(b);
+    rc = stage_outputs(b, true, false);
     if (rc != MMF_OK) return rc;
     const MmfDesc& d = b->desc[0];
     const size_t bytes = sizeof(double2) * (size_t)nt * d.D * d.D;
@@ -1617,13 +1617,8 @@ extern "C" int mmf_transition_avg_dev(mmf_sys* s, double* P, void* stream) {
     std::lock_guard<std::recursive_mutex> lk(s->ctx->mu);
     CU(cudaSetDevice(s->ctx->device));
     mmf_batch* b = s->solo;
-    if (b->last_stage < 3) {
-        if (b->nt > 0 && !b->times_set) {
-            std::vector<double> z((size_t)b->nt, 0.0);
-            int rc = mmf_batch_set_times(b, 0.0, z.data());
-            if (rc != MMF_OK) return rc;
-        }
-        int rc = stage_outputs(b);
+    if (!b->p_valid) {
+        int rc = stage_outputs(b, false, true);
         if (rc != MMF_OK) return rc;
     }
     const MmfDesc& d = b->desc[0];
