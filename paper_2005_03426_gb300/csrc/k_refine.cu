@@ -1123,60 +1123,72 @@ __global__ void __launch_bounds__(256) k_sort_pairs(const MmfDesc* __restrict__ 
 // (|G_ij| ~ eps32 before the first step, of the size of its second-order error after it), and a
 // cluster wider than the band meets G_ij ~ 0 outside it in the update; the cluster separation
 // then forms the cluster's own Gram matrix from X.  Only near pairs need G to FP64 accuracy.
-#define RF_BC 32            // columns per CTA
-#define RF_BR 16            // rows per staged chunk
+#define RF_BC 15            // columns per CTA: 15 x 17 pairs, one to a thread
+#define RF_BR 32            // rows per staged chunk
 
 // G = X^H X on the band |i - j| <= RF_W in double-FP32, written into the full n x n G (column-major,
-// ld); its other entries are left as they are (the update reads G only on the band then).
+// ld); its other entries are left as they are (the update reads G only on the band then).  X comes in
+// the FP32 pieces X1 + Xlo that the H_F product left (EXACT: the first step's X, which FP32 holds, so
+// products have no cross terms), and only pairs j >= i are formed, the mirror being the conjugate.
+// FP32 issue bounds it (32 instructions a complex product without cross terms, 44 with).  64 systems of
+// n = 1323: both pairs of every offset from FP64 X, split on the FP64 units in each CTA, 7.2 ms a
+// launch; this form 2.5 (first step) and 3.5 ms; one system 0.80 -> 0.15 and 0.19 ms.
+template <bool EXACT>
 __global__ void __launch_bounds__(256) k_gram_band_df32(const MmfDesc* __restrict__ descs,
                                                         const int* __restrict__ idx,
-                                                        const double2* __restrict__ Xg,
+                                                        const float2* __restrict__ X1g,
+                                                        const float2* __restrict__ Xlog,
                                                         double2* __restrict__ Gg) {
-    __shared__ Split xs[RF_BR][RF_BC + 2 * RF_W + 1];
+    constexpr int NC = RF_BC + RF_W;   // staged columns
+    __shared__ float2 x1s[RF_BR][NC + 2];
+    __shared__ float2 xls[EXACT ? 1 : RF_BR][NC + 2];
     const MmfDesc d = descs[idx[blockIdx.y]];
     const int n = d.n;
     const int i0 = blockIdx.x * RF_BC;
     if (i0 >= n) return;
-    const int cbase = i0 - RF_W;             // first staged column
-    const int ncs = RF_BC + 2 * RF_W;         // staged columns
-    const double2* X = Xg + d.mat_off;
-    // each thread owns up to 5 (i, j) pairs: pair p = tid + 256 q, i = i0 + p / BW, j = i + p % BW - W
-    DF gr[5], gi[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) gr[q] = gi[q] = DF{0.f, 0.f};
+    const float2* X1 = X1g + d.mat_off;
+    const float2* Xlo = EXACT ? nullptr : Xlog + d.mat_off;
+    const int ii = threadIdx.x / (RF_W + 1), off = threadIdx.x - ii * (RF_W + 1);
+    const bool own = ii < RF_BC;
+    DF gr = DF{0.f, 0.f}, gi = gr;
     for (int k0 = 0; k0 < n; k0 += RF_BR) {
-        for (int e = threadIdx.x; e < RF_BR * ncs; e += 256) {
+        for (int e = threadIdx.x; e < RF_BR * NC; e += 256) {
             const int c = e / RF_BR, kk = e - c * RF_BR;
-            const int col = cbase + c, k = k0 + kk;
-            const bool ok = k < n && col >= 0 && col < n;
-            xs[kk][c] = split(ok ? X[(int64_t)col * d.ld + k] : make_double2(0.0, 0.0));
+            const int col = i0 + c, k = k0 + kk;
+            const bool ok = k < n && col < n;
+            x1s[kk][c] = ok ? X1[(int64_t)col * d.ld + k] : make_float2(0.f, 0.f);
+            if (!EXACT) xls[kk][c] = ok ? Xlo[(int64_t)col * d.ld + k] : make_float2(0.f, 0.f);
         }
         __syncthreads();
+        if (own) {
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            const int p = threadIdx.x + 256 * q;
-            if (p < RF_BC * RF_BW) {
-                const int ii = p / RF_BW, off = p - ii * RF_BW;  // column i0+ii, partner i0+ii+off-W
-                const int cix = ii + RF_W, cj = ii + off;           // staged indices
-                for (int kk = 0; kk < RF_BR; ++kk) df_cmacc(gr[q], gi[q], xs[kk][cix], xs[kk][cj]);
-                df_renorm(gr[q]); df_renorm(gi[q]);
+            for (int h = 0; h < RF_BR; h += 16) {
+#pragma unroll 8
+                for (int kk = h; kk < h + 16; ++kk) {
+                    const float2 a = x1s[kk][ii], b = x1s[kk][ii + off];
+                    if (EXACT) {
+                        df_mac11(gr, a.x, b.x);
+                        df_mac11(gr, a.y, b.y);
+                        df_mac11(gi, a.x, b.y);
+                        df_mac11(gi, -a.y, b.x);
+                    } else {
+                        const float2 al = xls[kk][ii], bl = xls[kk][ii + off];
+                        df_cmacc(gr, gi, Split{a.x, al.x, a.y, al.y}, Split{b.x, bl.x, b.y, bl.y});
+                    }
+                }
+                df_renorm(gr);
+                df_renorm(gi);
             }
         }
         __syncthreads();
     }
-    double2* G = Gg + d.mat_off;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        const int p = threadIdx.x + 256 * q;
-        if (p < RF_BC * RF_BW) {
-            const int ii = p / RF_BW, off = p - ii * RF_BW;
-            const int i = i0 + ii, j = i + off - RF_W;
-            if (i < n && j >= 0 && j < n) {
-                double2 g = make_double2((double)gr[q].hi + (double)gr[q].lo, (double)gi[q].hi + (double)gi[q].lo);
-                if (i == j) g.y = 0.0;
-                G[(int64_t)j * d.ld + i] = g;
-            }
-        }
+    const int i = i0 + ii, j = i + off;
+    if (own && j < n) {
+        double2 g = df_value(gr, gi);
+        if (off == 0) g.y = 0.0;
+        double2* G = Gg + d.mat_off;
+        G[(int64_t)j * d.ld + i] = g;
+        if (off > 0) G[(int64_t)i * d.ld + j] = conj(g);
     }
 }
 
@@ -1209,12 +1221,11 @@ cudaError_t mmf_launch_coef_pattern(const MmfLaunch& L, const double2* coef, int
 }
 
 cudaError_t mmf_launch_refine_pre(const MmfLaunch& L, const float4* cs, const int* pat, const double2* X,
-                                  const double* lam0, double2* HX, double2* T, float2* X1, void* ops, void* jobs,
-                                  int* status, int second) {
+                                  const double* lam0, double2* HX, double2* T, float2* X1, float2* Xlo, void* ops,
+                                  void* jobs, int* status, int second) {
     if (L.count <= 0) return cudaSuccess;
-    // the first step's X holds FP32 eigenvectors (no remainder); the remainder of a second step's
-    // X goes to T, which is free until C is written
-    apply_hf(L, cs, pat, X, X1, second ? reinterpret_cast<float2*>(T) : nullptr, HX);
+    // the first step's X holds FP32 eigenvectors (no remainder)
+    apply_hf(L, cs, pat, X, X1, second ? Xlo : nullptr, HX);
     k_w_prep_B<<<dim3(512, L.count), 256, 0, L.stream>>>(L.desc, L.idx, X, HX, lam0, ops);
     k_w_prep_A<<<dim3(256, L.count), 256, 0, L.stream>>>(L.desc, L.idx, X1, ops);
     k_w_jobs<<<(L.count + 127) / 128, 128, 0, L.stream>>>(L.desc, L.idx, L.count, ops, T, 0, (Tf3Job*)jobs);
@@ -1265,9 +1276,11 @@ cudaError_t mmf_launch_refine_update(const MmfLaunch& L, const double2* coef, co
     return cudaGetLastError();
 }
 
-cudaError_t mmf_launch_refine_band_g(const MmfLaunch& L, const double2* X, double2* G) {
+cudaError_t mmf_launch_refine_band_g(const MmfLaunch& L, const float2* X1, const float2* Xlo, double2* G) {
     if (L.count <= 0) return cudaSuccess;
-    k_gram_band_df32<<<dim3((L.nmax + RF_BC - 1) / RF_BC, L.count), 256, 0, L.stream>>>(L.desc, L.idx, X, G);
+    const dim3 g((L.nmax + RF_BC - 1) / RF_BC, L.count);
+    if (Xlo) k_gram_band_df32<false><<<g, 256, 0, L.stream>>>(L.desc, L.idx, X1, Xlo, G);
+    else k_gram_band_df32<true><<<g, 256, 0, L.stream>>>(L.desc, L.idx, X1, nullptr, G);
     return cudaGetLastError();
 }
 

@@ -1149,28 +1149,30 @@ static int stage_eig(mmf_batch* b) {
         MmfLaunch La = launch_of(b, b->all, b->d_all, b->nmax_all);
         LAUNCH(mmf_launch_refine_split_coef(b->d_coef, b->d_coefs, b->n_coef, b->stream), 1);
         LAUNCH(mmf_launch_coef_pattern(La, b->d_coef, b->d_pat), 1);
-        LAUNCH(mmf_launch_refine_pre(La, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, b->d_oz, b->d_jobs,
-                                     b->d_status, 0),
+        LAUNCH(mmf_launch_refine_pre(La, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, nullptr, b->d_oz,
+                                     b->d_jobs, b->d_status, 0),
                6);
         mark(b, ST_GRAM);
         // the first step needs G = X^H X only on the band |i - j| <= 16 (far pairs enter its update
         // through C), as the hybrid second step does
-        LAUNCH(mmf_launch_refine_band_g(La, b->d_Zf, b->d_R), 1);
+        LAUNCH(mmf_launch_refine_band_g(La, b->d_X1, nullptr, b->d_R), 1);
         mark(b, ST_REFINE2);
         // every system takes a second step (hybrid or full) below, so the first one applies the
         // near band of Et in FP32
         LAUNCH(mmf_launch_refine_update(La, b->d_coef, b->d_pat, b->d_Zf, b->d_X1, b->d_E, b->d_R, b->d_HX, b->d_T, b->d_E2,
                                         b->d_status, b->d_cid, b->d_oz, b->d_jobs, b->d_Eb, 1, 1),
                9);
+        // the second step's FP32 remainder of X, in a pool that only the final sort writes
+        float2* const Xlo = reinterpret_cast<float2*>(b->d_S);
         // second step from lam0 = the first step's eigenvalues (E is rewritten at the end)
         CU(cudaMemcpyAsync(b->d_E, b->d_E2, sizeof(double) * b->n_vec, cudaMemcpyDeviceToDevice, b->stream));
         if (!b->rband.empty()) {
             // hybrid: C = X1^H W for all pairs on the tensor cores, G only on the band
             MmfLaunch Lb = launch_of(b, b->rband, b->d_rband, b->nmax_rband);
-            LAUNCH(mmf_launch_refine_pre(Lb, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, b->d_oz,
+            LAUNCH(mmf_launch_refine_pre(Lb, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, Xlo, b->d_oz,
                                          b->d_jobs, b->d_status, 2),
                    6);
-            LAUNCH(mmf_launch_refine_band_g(Lb, b->d_Zf, b->d_R), 1);
+            LAUNCH(mmf_launch_refine_band_g(Lb, b->d_X1, Xlo, b->d_R), 1);
             LAUNCH(mmf_launch_refine_update(Lb, b->d_coef, b->d_pat, b->d_Zf, b->d_X1, b->d_E, b->d_R, b->d_HX, b->d_T,
                                             b->d_E2, b->d_status, b->d_cid, b->d_oz, b->d_jobs, b->d_Eb, 0, 1),
                    9);
@@ -1178,7 +1180,7 @@ static int stage_eig(mmf_batch* b) {
         if (!b->rfull.empty()) {
             // full second step: G of the FP64 iterate as G(X1) + C' + C'^H
             MmfLaunch Lf = launch_of(b, b->rfull, b->d_rfull, b->nmax_rfull);
-            LAUNCH(mmf_launch_refine_pre(Lf, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, b->d_oz,
+            LAUNCH(mmf_launch_refine_pre(Lf, b->d_coefs, b->d_pat, b->d_Zf, b->d_E, b->d_HX, b->d_T, b->d_X1, Xlo, b->d_oz,
                                          b->d_jobs, b->d_status, 1),
                    9);
             LAUNCH(refine_gram(b, Lf, 1), 3);

@@ -314,7 +314,7 @@ cudaError_t mmf_launch_micromotion(const MmfLaunch& L, int D, const double2* Z, 
 cudaError_t mmf_launch_refine_split_coef(const double2* coef, float4* cs, int64_t count, cudaStream_t st);
 cudaError_t mmf_launch_coef_pattern(const MmfLaunch& L, const double2* coef, int* pat);
 cudaError_t mmf_launch_refine_pre(const MmfLaunch& L, const float4* cs, const int* pat, const double2* X, const double* lam0,
-                                  double2* HX, double2* T, float2* X1, void* ops, void* jobs, int* status,
+                                  double2* HX, double2* T, float2* X1, float2* Xlo, void* ops, void* jobs, int* status,
                                   int second);
 cudaError_t mmf_launch_refine_gram(const MmfLaunch& L, const float2* X1, double2* G, const double2* T, int second);
 cudaError_t mmf_launch_refine_gram_fix(const MmfLaunch& L, double2* G, const double2* T);
@@ -327,7 +327,8 @@ cudaError_t mmf_launch_refine_update(const MmfLaunch& L, const double2* coef, co
                                      int band_fp32, int g_band);
 // first step and hybrid second step: G = X^H X on the band |i - j| <= 16 (double-FP32), the rest
 // of G left unset (the update then runs with g_band = 1)
-cudaError_t mmf_launch_refine_band_g(const MmfLaunch& L, const double2* X, double2* G);
+// (X in the FP32 pieces mmf_launch_refine_pre left; Xlo null: X1 alone)
+cudaError_t mmf_launch_refine_band_g(const MmfLaunch& L, const float2* X1, const float2* Xlo, double2* G);
 cudaError_t mmf_launch_refine_finish(const MmfLaunch& L, double2* X, double* E, const double* lam, double2* S,
                                      int64_t mat_elems);
 // Gram product on the BF16 tensor cores by exact integer slicing (k_ozaki.cu)
