@@ -211,15 +211,15 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
 // step's vectors are known, so a sweep follows its predecessor by a step and the part of a step up to
 // there, with its loads and B v_p done beforehand, where it waited for two whole steps (one FP32 system
 // of n = 1323 15.1 -> 13.2 ms, eight in FP64 99 -> 87).  With few groups per system (CL <= 2 and wide
-// windows) the SMs are busy anyway and the publication's fence costs 5 %: there a sweep waits for all of
-// the predecessor's step s + 1.
+// windows) the SMs are busy anyway (64 systems: 25.0 ms with the publication, 25.2 without): there a sweep
+// waits for all of the predecessor's step s + 1.
 //
 // What bounds it: the critical path of one sweep after another (about 1.5 n steps), so the latency of a
 // step; on the FP64 path the 2 FP64 FMAs per clock
 // of an SM (24 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
 // CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
 // b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
-// kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
+// kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 25.2 ms; eight systems in FP64
 // 455 -> 87 ms.
 //
 // CL = 1: one CTA per system.  CL > 1: a cluster of CL CTAs per system, the sweeps dealt round-robin
@@ -821,7 +821,7 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
 
 // The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
 // pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
-// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
+// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 25 ms that 64 such systems
 // take, with 8 it takes 13.2.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
