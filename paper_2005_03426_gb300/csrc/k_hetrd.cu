@@ -490,6 +490,10 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
         T.tmem = tc_tmem;
     }
 
+    // The first column pushes into the partners' shared memory: every CTA of the cluster has to be running
+    // before any of them does.
+    if (CL > 1) cluster.sync();
+
     // Rows in chunks of 32, chunk q with CTA q % CL.  In the O(m i) steps the warps split into CG
     // groups over the panel's columns, each group's NCW warps over this CTA's chunks.
     constexpr int CG = CL >= 6 ? 4 : CL >= 4 ? 2 : 1;

@@ -1,0 +1,43 @@
+"""Ordering rules that the kernels have to keep whatever the hardware happens to do, read off the
+sources (breaking one is not something a GPU may be made to show)."""
+
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2005_03426_gb300", "csrc")
+
+
+def _source(name):
+    """The file without its comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def _block(text, at):
+    """The brace-delimited block that opens at or after position `at`."""
+    i = text.index("{", at)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return text[i:j + 1]
+    raise ValueError("unbalanced braces")
+
+
+def _kernels(name):
+    text = _source(name)
+    for m in re.finditer(r"__global__\s+void(?:\s+__launch_bounds__\((?:[^()]|\([^()]*\))*\))?\s*(\w+)\s*\(", text):
+        body = _block(text, m.end())
+        yield m.group(1), text[m.end():text.index(body, m.end())], body
+
+
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cu")))
+def test_cluster_has_started_before_a_partner_is_addressed(name):
+    """A CTA may access a partner's shared memory only once the whole cluster is running: the first
+    cluster-wide barrier comes before the first access."""
+    for kernel, _, body in _kernels(name):
+        first = min((body.index(w) for w in ("map_shared_rank", "key_load(", "flag_load(") if w in body), default=None)
+        if first is not None:
+            assert "cluster.sync()" in body[:first], kernel
