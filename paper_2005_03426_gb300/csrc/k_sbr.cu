@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             }
         }
         stopped = __shfl_sync(0xffffffffu, stopped, 0);
+        __syncwarp();  // orders the other lanes' loads after lane 0's acquire (a shuffle orders no memory)
     };
     for (int j = gg; j <= n - 2; j += NGT) {
         const int nsteps = (n - 2 - j) / b + 1;

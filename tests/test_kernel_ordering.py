@@ -41,3 +41,13 @@ def test_cluster_has_started_before_a_partner_is_addressed(name):
         first = min((body.index(w) for w in ("map_shared_rank", "key_load(", "flag_load(") if w in body), default=None)
         if first is not None:
             assert "cluster.sync()" in body[:first], kernel
+
+
+def test_a_warp_loads_after_its_lanes_acquire():
+    """Where one lane polls a progress key for its warp, a warp barrier follows the poll: the lanes'
+    loads are ordered after the acquire by it alone (a shuffle orders no memory)."""
+    text = _source("k_sbr.cu")
+    at = text.index("auto wait_for")
+    body = _block(text, text.index(")", at))
+    assert "key_load(" in body and "__syncwarp()" in body[body.index("key_load("):]
+    assert text.count("key_load(") == 2  # its definition and this poll
