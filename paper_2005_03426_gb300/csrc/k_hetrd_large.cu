@@ -37,6 +37,9 @@ struct LgScalars {     // per-column scalars shared between the launches (device
 
 // Programmatic stream serialisation: a kernel may be started before its predecessor on the stream has
 // finished; lg_wait returns once it has (all of its writes visible), lg_go lets the successor start.
+// What a kernel reads is thus written while it already runs, up to its lg_wait: no pointer here may be
+// declared __restrict__ (data unchanged for the kernel's whole life, which allows read-only loads and loads
+// ahead of the wait).
 __device__ __forceinline__ void lg_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void lg_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 static_assert(sizeof(LgScalars) <= 8 * sizeof(double), "the scalars fit the system's 8-double auxiliary slot");
@@ -78,13 +81,13 @@ __device__ __forceinline__ C lg_alpha2(const LgScalars* sc) {
 // CTA forms the reflector (one thread) and clears the sums of the column's later steps.  vbuf still
 // holds the previous column's v (from row k on).
 template <class R>
-__global__ void __launch_bounds__(LG_B) k_lg_colupd(typename Cx<R>::T* __restrict__ A, int n, int ld, int k, int i,
-                                                    const typename Cx<R>::T* __restrict__ V,
-                                                    typename Cx<R>::T* __restrict__ W,
-                                                    const typename Cx<R>::T* __restrict__ vbuf,
-                                                    typename Cx<R>::T* __restrict__ xbuf, LgScalars* sc,
-                                                    double* __restrict__ dd, double* __restrict__ ee,
-                                                    typename Cx<R>::T* __restrict__ tau) {
+__global__ void __launch_bounds__(LG_B) k_lg_colupd(typename Cx<R>::T* A, int n, int ld, int k, int i,
+                                                    const typename Cx<R>::T* V,
+                                                    typename Cx<R>::T* W,
+                                                    const typename Cx<R>::T* vbuf,
+                                                    typename Cx<R>::T* xbuf, LgScalars* sc,
+                                                    double* dd, double* ee,
+                                                    typename Cx<R>::T* tau) {
     typedef typename Cx<R>::T C;
     __shared__ C wk[MMF_NB], vk[MMF_NB], ps[LG_G - 1][LG_R];
     __shared__ R red[33];
@@ -94,30 +97,37 @@ __global__ void __launch_bounds__(LG_B) k_lg_colupd(typename Cx<R>::T* __restric
     lg_go();
     const C a2 = i > 0 ? lg_alpha2<C, R>(sc) : czero<C>();
     if (tid < i) {
-        C w = W[k + (int64_t)tid * ld];
         const C v = V[k + (int64_t)tid * ld];
-        // (row k of W(:, i - 1) is this kernel's own first row: from its uncorrected copy in W(k, NB))
-        if (tid == i - 1) w = xbuf[2 * MMF_NB] + a2 * v;
+        // (row k of W(:, i - 1) is corrected by the first CTA of this launch: from its uncorrected copy)
+        const C w = tid == i - 1 ? xbuf[2 * MMF_NB] + a2 * v : W[k + (int64_t)tid * ld];
         wk[tid] = conj(w);
         vk[tid] = conj(v);
     }
     __syncthreads();
-    // thread (row, g): columns g, g + LG_G, ... of the panel
+    // thread (row, g): columns g, g + LG_G, ... of the panel, all of them loaded before the one store
     const int rl = tid & (LG_R - 1), g = tid / LG_R, r = k + blockIdx.x * LG_R + rl;
     C acc = czero<C>(), acc2 = czero<C>(), x = czero<C>();
     if (r < n) {
+        constexpr int NU = MMF_NB / LG_G;
+        C w[NU], v[NU], vp = czero<C>();
         if (g == 0) x = A[(int64_t)k * ld + r];
+        if (i > 0) vp = vbuf[r - k];
 #pragma unroll
-        for (int u = 0; u < MMF_NB / LG_G; ++u) {
+        for (int u = 0; u < NU; ++u) {
+            const int c = g + u * LG_G;
+            w[u] = c < i ? W[r + (int64_t)c * ld] : czero<C>();
+            v[u] = c < i ? V[r + (int64_t)c * ld] : czero<C>();
+        }
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
             const int c = g + u * LG_G;
             if (c < i) {
-                C w = W[r + (int64_t)c * ld];
                 if (c == i - 1) {
-                    w = w + a2 * vbuf[r - k];
-                    W[r + (int64_t)c * ld] = w;
+                    w[u] = w[u] + a2 * vp;
+                    W[r + (int64_t)c * ld] = w[u];
                 }
-                acc = cmac(acc, V[r + (int64_t)c * ld], wk[c]);
-                acc2 = cmac(acc2, w, vk[c]);
+                acc = cmac(acc, v[u], wk[c]);
+                acc2 = cmac(acc2, w[u], vk[c]);
             }
         }
     }
@@ -175,12 +185,12 @@ __global__ void __launch_bounds__(LG_B) k_lg_colupd(typename Cx<R>::T* __restric
 // (2) v from column k over the grid (rows of this CTA): A(r, k) <- v_r below the subdiagonal,
 // V(:, i), vbuf, y = 0; then the CTA's parts of x_w = W^H v and x_v = V^H v (warp per product)
 template <class R>
-__global__ void __launch_bounds__(LG_B) k_lg_vscale(typename Cx<R>::T* __restrict__ A, int n, int ld, int k, int i,
-                                                    typename Cx<R>::T* __restrict__ V,
-                                                    const typename Cx<R>::T* __restrict__ W,
-                                                    typename Cx<R>::T* __restrict__ vbuf,
-                                                    typename Cx<R>::T* __restrict__ ybuf,
-                                                    typename Cx<R>::T* __restrict__ xbuf, const LgScalars* sc) {
+__global__ void __launch_bounds__(LG_B) k_lg_vscale(typename Cx<R>::T* A, int n, int ld, int k, int i,
+                                                    typename Cx<R>::T* V,
+                                                    const typename Cx<R>::T* W,
+                                                    typename Cx<R>::T* vbuf,
+                                                    typename Cx<R>::T* ybuf,
+                                                    typename Cx<R>::T* xbuf, const LgScalars* sc) {
     typedef typename Cx<R>::T C;
     __shared__ C vs[LG_R];
     const int tid = threadIdx.x, r0 = blockIdx.x * LG_R, r = r0 + tid;
@@ -245,9 +255,9 @@ __global__ void __launch_bounds__(LG_B) k_lg_vscale(typename Cx<R>::T* __restric
 // memory over the block's four warps of that half.
 #define LG_HB 128
 template <class R>
-__global__ void __launch_bounds__(256) k_lg_hemv(const typename Cx<R>::T* __restrict__ A, int n, int ld, int k,
-                                                 const typename Cx<R>::T* __restrict__ vbuf,
-                                                 typename Cx<R>::T* __restrict__ ybuf) {
+__global__ void __launch_bounds__(256) k_lg_hemv(const typename Cx<R>::T* A, int n, int ld, int k,
+                                                 const typename Cx<R>::T* vbuf,
+                                                 typename Cx<R>::T* ybuf) {
     typedef typename Cx<R>::T C;
     __shared__ C vr_s[LG_HB], vc_s[LG_HB];
     __shared__ C colsum[4][LG_HB];  // [warp within the half][column]
@@ -353,11 +363,11 @@ __global__ void __launch_bounds__(256) k_lg_hemv(const typename Cx<R>::T* __rest
 // xbuf[2 NB], where the next column's CTAs read it while its owner corrects W
 template <class R>
 __global__ void __launch_bounds__(LG_B) k_lg_w(int n, int ld, int k, int i,
-                                               const typename Cx<R>::T* __restrict__ V,
-                                               typename Cx<R>::T* __restrict__ W,
-                                               const typename Cx<R>::T* __restrict__ vbuf,
-                                               const typename Cx<R>::T* __restrict__ ybuf,
-                                               typename Cx<R>::T* __restrict__ xbuf, LgScalars* sc) {
+                                               const typename Cx<R>::T* V,
+                                               typename Cx<R>::T* W,
+                                               const typename Cx<R>::T* vbuf,
+                                               const typename Cx<R>::T* ybuf,
+                                               typename Cx<R>::T* xbuf, LgScalars* sc) {
     typedef typename Cx<R>::T C;
     __shared__ C xs[2 * MMF_NB], ps[LG_G - 1][LG_R];
     __shared__ R red[33];
@@ -398,8 +408,8 @@ __global__ void __launch_bounds__(LG_B) k_lg_w(int n, int ld, int k, int i,
 
 // the last correction of a panel's last column, W(:, i) += alpha2 v below row k
 template <class R>
-__global__ void __launch_bounds__(LG_B) k_lg_w2(int n, int ld, int k, int i, typename Cx<R>::T* __restrict__ W,
-                                                const typename Cx<R>::T* __restrict__ vbuf, const LgScalars* sc) {
+__global__ void __launch_bounds__(LG_B) k_lg_w2(int n, int ld, int k, int i, typename Cx<R>::T* W,
+                                                const typename Cx<R>::T* vbuf, const LgScalars* sc) {
     typedef typename Cx<R>::T C;
     lg_wait();
     lg_go();
@@ -411,9 +421,9 @@ __global__ void __launch_bounds__(LG_B) k_lg_w2(int n, int ld, int k, int i, typ
 // the diagonal (the diagonal tiles masked to r >= c), the panel's columns staged 8 at a time
 #define LG_KC 8
 template <class R>
-__global__ void __launch_bounds__(256) k_lg_her2k(typename Cx<R>::T* __restrict__ A, int n, int ld, int c0, int nb,
-                                                  const typename Cx<R>::T* __restrict__ V,
-                                                  const typename Cx<R>::T* __restrict__ W) {
+__global__ void __launch_bounds__(256) k_lg_her2k(typename Cx<R>::T* A, int n, int ld, int c0, int nb,
+                                                  const typename Cx<R>::T* V,
+                                                  const typename Cx<R>::T* W) {
     typedef typename Cx<R>::T C;
     __shared__ C tVr[LG_KC][LG_TILE], tWr[LG_KC][LG_TILE], tVc[LG_KC][LG_TILE], tWc[LG_KC][LG_TILE];
     const int rbase = c0 + blockIdx.x * LG_TILE, cbase = c0 + blockIdx.y * LG_TILE;

@@ -51,3 +51,13 @@ def test_a_warp_loads_after_its_lanes_acquire():
     body = _block(text, text.index(")", at))
     assert "key_load(" in body and "__syncwarp()" in body[body.index("key_load("):]
     assert text.count("key_load(") == 2  # its definition and this poll
+
+
+def test_programmatically_serialised_kernels_assume_no_constant_inputs():
+    """A kernel that may start before its predecessor has finished (griddepcontrol.wait) runs while its
+    inputs are written: none of its pointers is __restrict__, which promises the compiler that they do
+    not change and permits read-only loads."""
+    found = [(k, args) for k, args, body in _kernels("k_hetrd_large.cu") if "lg_wait()" in body]
+    assert len(found) == 6
+    for kernel, args in found:
+        assert "__restrict__" not in args, kernel
