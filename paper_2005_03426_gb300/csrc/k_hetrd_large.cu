@@ -517,7 +517,7 @@ static cudaError_t run_large(typename Cx<R>::T* A, int n, int ld, typename Cx<R>
 }
 
 // One large system (host-side descriptor copy `d`, device pointers into the batch pools).
-// work: 3 n + 2 NB + 1 complex elements of the working precision; sc: one LgScalars.
+// work: 2 n + 2 NB + 1 complex elements of the working precision, aligned to one; sc: one LgScalars.
 cudaError_t mmf_launch_hetrd_large(const MmfDesc& d, void* H, void* Vp, void* Wp, double* dvec, double* evec,
                                    void* tau, void* work, void* sc, int fp32, cudaStream_t st) {
     if (fp32)

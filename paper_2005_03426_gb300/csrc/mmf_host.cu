@@ -1122,7 +1122,10 @@ static int stage_eig(mmf_batch* b) {
         }
         for (int i : b->huge) {  // one system at a time over the whole GPU
             const MmfDesc& d = b->desc[i];
-            void* work = (void*)(b->d_Y + d.sq_off);
+            // its vectors lie in the system's eigenvector slot, which is free until the back-transform, begins on
+            // a 16-byte boundary and holds n x ld >= 36 n complex elements (a slot of Y is 8-byte aligned: an
+            // odd number of doubles may precede it)
+            void* work = (void*)(b->d_Zf + d.mat_off);
             void* sc = (void*)(b->d_aux + 8 * i);
             LAUNCH(mmf_launch_hetrd_large(d, b->d_H, b->d_Vp, b->d_Wp, b->d_d, b->d_e, b->d_tau, work, sc, fp32,
                                           b->stream),
