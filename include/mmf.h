@@ -74,6 +74,11 @@ MMF_API int mmf_ctx_destroy(mmf_ctx* ctx);
 /* Device bytes currently held by the context's batches. */
 MMF_API size_t mmf_ctx_bytes_in_use(const mmf_ctx* ctx);
 MMF_API size_t mmf_ctx_budget(const mmf_ctx* ctx);
+/* Streams the context has made beside the one it works on: a batch whose systems take several solver
+ * paths runs them side by side, forked from and joined into its own stream.  Returns their number and
+ * puts up to `cap` of them (cudaStream_t) into `streams`.  At most 7 for the context's stream and for
+ * each slot of a server, whatever the number of batches. */
+MMF_API int mmf_ctx_side_streams(mmf_ctx* ctx, void** streams, int cap);
 /* Size thresholds of the solver paths for batches created afterwards (value < 0 restores the
  * default): MMF_OPT_JACOBI_N_FP64 / _MIXED: largest n solved by the shared-memory Jacobi kernel
  * (defaults 84 / 118, also the maxima; values below 4 act as 4); MMF_OPT_LARGE_N: smallest n reduced by the whole-GPU

@@ -46,6 +46,16 @@ struct TuneRule {
     int jacobi, band, bt_tc;
 };
 
+// Side streams for the solver paths of a mixed batch (Branches), of one stream that plans run on: the
+// context's or a serving slot's.  All plans of that stream share them (their work is in order anyway), so
+// their number does not grow with the plans, resident ones of a server included.
+struct SideStreams {
+    cudaStream_t main = nullptr;
+    cudaEvent_t fork = nullptr;
+    std::vector<cudaStream_t> st;
+    std::vector<cudaEvent_t> done;  // done[i]: end of st[i]'s branch
+};
+
 struct mmf_ctx {
     int device = 0;
     std::vector<TuneRule> rules;     // first match wins
@@ -60,6 +70,7 @@ struct mmf_ctx {
     int64_t jacobi_sweeps = -1;      // Jacobi sweep cap; -1 = library default
     int64_t band_max = -1;           // largest half-bandwidth reduced by the bulge chase; -1 = default
     int64_t hetrd_tc = -1;           // mixed path: dense reduction's trailing update on the tensor cores
+    std::vector<SideStreams> side;
     cudaEvent_t order_ev = nullptr;  // orders the context stream against callers' streams (*_dev calls)
     std::recursive_mutex mu;
 };
@@ -154,9 +165,7 @@ struct mmf_batch {
     // per-stage CUDA-event timing (optional)
     int timing_runs = 0, runs_recorded = 0;
     std::vector<cudaEvent_t> ev;
-    // side streams for the solver paths of a mixed batch (run_branches); empty if it has one path
-    std::vector<cudaStream_t> side;
-    std::vector<cudaEvent_t> side_ev;  // side_ev[i]: end of side[i]'s branch; the last one: the fork
+    int nside = 0;  // side streams it uses: its solver paths beyond the first
     // CUDA graph of the whole run (optional)
     bool use_graph = false;
     cudaGraphExec_t graph_exec = nullptr;
@@ -326,9 +335,59 @@ extern "C" int mmf_ctx_create(int device, size_t budget, void* stream, mmf_ctx**
     return MMF_OK;
 }
 
+// The side streams of `main`, at least n of them (under the context's lock; not during a capture, since
+// missing ones are created).
+static cudaError_t side_streams(mmf_ctx* c, cudaStream_t main, int n, SideStreams** out) {
+    SideStreams* s = nullptr;
+    for (SideStreams& q : c->side)
+        if (q.main == main) s = &q;
+    if (!s) {
+        SideStreams q;
+        q.main = main;
+        cudaError_t e = cudaEventCreateWithFlags(&q.fork, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        c->side.push_back(q);
+        s = &c->side.back();
+    }
+    while ((int)s->st.size() < n) {
+        cudaStream_t st = nullptr;
+        cudaEvent_t ev = nullptr;
+        cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            cudaStreamDestroy(st);
+            return e;
+        }
+        s->st.push_back(st);
+        s->done.push_back(ev);
+    }
+    *out = s;
+    return cudaSuccess;
+}
+
+static void destroy_side(SideStreams& s) {
+    for (cudaStream_t st : s.st) cudaStreamDestroy(st);
+    for (cudaEvent_t e : s.done) cudaEventDestroy(e);
+    cudaEventDestroy(s.fork);
+}
+
+extern "C" int mmf_ctx_side_streams(mmf_ctx* c, void** streams, int cap) {
+    if (!c || cap < 0 || (cap > 0 && !streams)) return fail(MMF_ERR_ARG, "ctx and streams required");
+    std::lock_guard<std::recursive_mutex> lk(c->mu);
+    int n = 0;
+    for (const SideStreams& s : c->side)
+        for (cudaStream_t st : s.st) {
+            if (n < cap) streams[n] = st;
+            ++n;
+        }
+    return n;
+}
+
 extern "C" int mmf_ctx_destroy(mmf_ctx* c) {
     if (!c) return MMF_ERR_ARG;
     cudaSetDevice(c->device);
+    for (SideStreams& s : c->side) destroy_side(s);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     if (c->order_ev) cudaEventDestroy(c->order_ev);
     delete c;
@@ -498,15 +557,7 @@ static void fill_coef(const mmf_batch* b, double2* dst) {
     }
 }
 
-static void drop_side_streams(mmf_batch* b) {
-    for (cudaEvent_t e : b->side_ev) cudaEventDestroy(e);
-    for (cudaStream_t st : b->side) cudaStreamDestroy(st);
-    b->side_ev.clear();
-    b->side.clear();
-}
-
 static void free_batch_memory(mmf_batch* b) {
-    drop_side_streams(b);  // (their last work was joined into the batch's stream)
     if (b->base) {
         cudaFreeAsync(b->base, b->stream);
         b->ctx->used -= b->bytes;
@@ -876,17 +927,9 @@ static int batch_create(mmf_ctx* ctx, int count, mmf_sys* const* systems, int pr
     int nred = !b->medium.empty() + !b->tiny.empty(), nback = !b->bts.empty() + !b->btc.empty() + !b->btt.empty();
     for (int ci = 0; ci < 4; ++ci) nred += !b->sbr[ci].empty();
     for (int ci = 0; ci < 5; ++ci) nback += !b->sbt[ci].empty();
-    const int nside = std::max(nred, nback) - 1;
-    for (int i = 0; i < nside && e == cudaSuccess; ++i) {
-        cudaStream_t ss = nullptr;
-        e = cudaStreamCreateWithFlags(&ss, cudaStreamNonBlocking);
-        if (e == cudaSuccess) b->side.push_back(ss);
-    }
-    for (int i = 0; i <= nside && nside > 0 && e == cudaSuccess; ++i) {
-        cudaEvent_t ev = nullptr;
-        e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-        if (e == cudaSuccess) b->side_ev.push_back(ev);
-    }
+    b->nside = std::max(std::max(nred, nback) - 1, 0);
+    SideStreams* side = nullptr;
+    if (b->nside > 0) e = side_streams(ctx, b->stream, b->nside, &side);
     if (e != cudaSuccess) {
         free_batch_memory(b);
         delete b;
@@ -1030,21 +1073,29 @@ static cudaError_t refine_gram(mmf_batch* b, const MmfLaunch& L, int second) {
 // other streams' waits included) is ordered after all of them, also when a launch fails.
 struct Branches {
     mmf_batch* b;
+    SideStreams* side = nullptr;
     int used = 0;
     cudaError_t err = cudaSuccess;
     explicit Branches(mmf_batch* b_) : b(b_) {
-        if (!b->side.empty()) err = cudaEventRecord(b->side_ev.back(), b->stream);
+        if (b->nside > 0) err = side_streams(b->ctx, b->stream, b->nside, &side);
+        if (side && err == cudaSuccess) err = cudaEventRecord(side->fork, b->stream);
     }
+    // the next branch's stream (after an error the batch's own, so that nothing is left to join)
     cudaStream_t next() {
-        const int i = used++;
-        if (i == 0) return b->stream;
-        if (err == cudaSuccess) err = cudaStreamWaitEvent(b->side[i - 1], b->side_ev.back(), 0);
-        return b->side[i - 1];
+        if (used == 0 || err != cudaSuccess) {
+            used += used == 0;
+            return b->stream;
+        }
+        const int i = used - 1;
+        err = cudaStreamWaitEvent(side->st[i], side->fork, 0);
+        if (err != cudaSuccess) return b->stream;
+        ++used;
+        return side->st[i];
     }
     cudaError_t join() {
         for (int i = 0; i + 1 < used; ++i) {
-            cudaError_t e = cudaEventRecord(b->side_ev[i], b->side[i]);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->side_ev[i], 0);
+            cudaError_t e = cudaEventRecord(side->done[i], side->st[i]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, side->done[i], 0);
             if (err == cudaSuccess) err = e;
         }
         return err;
@@ -1245,6 +1296,8 @@ extern "C" int mmf_batch_run(mmf_batch* b) {
     g_launches = 0;
     if (!b->use_graph) return run_stages(b);
     if (!b->graph_exec) {
+        SideStreams* side = nullptr;  // (made before the capture: a plan may have come from another stream)
+        if (b->nside > 0) CU(side_streams(b->ctx, b->stream, b->nside, &side));
         // capture the whole launch sequence once; timing events (if on) record into slot 0
         const int saved = b->runs_recorded;
         b->runs_recorded = 0;
@@ -2210,6 +2263,17 @@ extern "C" int mmf_serve_destroy(mmf_server* sv) {
     for (CachedPlan& cp : sv->cache) mmf_batch_destroy(cp.b);
     sv->cache.clear();
     if (sv->park) cudaStreamDestroy(sv->park);
+    {  // the slots' side streams
+        std::lock_guard<std::recursive_mutex> lk(sv->ctx->mu);
+        auto& side = sv->ctx->side;
+        for (const Slot& sl : sv->slots)
+            for (size_t i = 0; i < side.size(); ++i)
+                if (side[i].main == sl.stream) {
+                    destroy_side(side[i]);
+                    side.erase(side.begin() + i);
+                    break;
+                }
+    }
     for (Slot& sl : sv->slots) {
         cudaStreamDestroy(sl.stream);
         cudaEventDestroy(sl.done);

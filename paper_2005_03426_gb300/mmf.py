@@ -80,6 +80,7 @@ _SIGS = {
     "mmf_ctx_destroy": (_I, [_P]),
     "mmf_ctx_bytes_in_use": (_SZ, [_P]),
     "mmf_ctx_budget": (_SZ, [_P]),
+    "mmf_ctx_side_streams": (_I, [_P, _PP, _I]),
     "mmf_ctx_set_option": (_I, [_P, _I, _I64]),
     "mmf_ctx_add_rule": (_I, [_P, _I, _I64, _I64, _I, _I, _I, _I, _I]),
     "mmf_ctx_clear_rules": (_I, [_P]),
@@ -233,6 +234,14 @@ class Context:
 
     def budget(self) -> int:
         return int(lib().mmf_ctx_budget(self.h))
+
+    def side_streams(self) -> List[int]:
+        """The streams (cudaStream_t) the context has made for solver paths that run side by side."""
+        buf = (ctypes.c_void_p * 1024)()
+        n = lib().mmf_ctx_side_streams(self.h, buf, 1024)
+        if n < 0:
+            _check(n)
+        return [int(buf[i]) for i in range(min(n, 1024))]
 
     def add_rule(self, precision: int, n_lo: int, n_hi: int, band_lo: int, band_hi: int,
                  jacobi: int = -1, band: int = -1, bt_tc: int = -1):
