@@ -75,8 +75,8 @@ MMF_API int mmf_ctx_destroy(mmf_ctx* ctx);
 MMF_API size_t mmf_ctx_bytes_in_use(const mmf_ctx* ctx);
 MMF_API size_t mmf_ctx_budget(const mmf_ctx* ctx);
 /* Streams the context has made beside the one it works on: a batch whose systems take several solver
- * paths runs them side by side, forked from and joined into its own stream.  Returns their number and
- * puts up to `cap` of them (cudaStream_t) into `streams`.  At most 7 for the context's stream and for
+ * paths runs them side by side, forked from and joined into its own stream and of that stream's
+ * priority.  Returns their number and puts up to `cap` of them (cudaStream_t) into `streams`.  At most 7 for the context's stream and for
  * each slot of a server, whatever the number of batches. */
 MMF_API int mmf_ctx_side_streams(mmf_ctx* ctx, void** streams, int cap);
 /* Size thresholds of the solver paths for batches created afterwards (value < 0 restores the

@@ -52,7 +52,7 @@ struct TuneRule {
 struct SideStreams {
     cudaStream_t main = nullptr;
     cudaEvent_t fork = nullptr;
-    std::vector<cudaStream_t> st;
+    std::vector<cudaStream_t> st;   // of main's priority
     std::vector<cudaEvent_t> done;  // done[i]: end of st[i]'s branch
 };
 
@@ -352,7 +352,9 @@ static cudaError_t side_streams(mmf_ctx* c, cudaStream_t main, int n, SideStream
     while ((int)s->st.size() < n) {
         cudaStream_t st = nullptr;
         cudaEvent_t ev = nullptr;
-        cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        int prio = 0;
+        cudaError_t e = cudaStreamGetPriority(main, &prio);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, prio);
         if (e != cudaSuccess) return e;
         e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
         if (e != cudaSuccess) {

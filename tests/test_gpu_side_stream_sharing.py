@@ -1,6 +1,6 @@
 """The side streams on which a batch's solver paths run beside one another: plans of one stream share
 them, so that their number does not grow with the plans (resident ones of a server included), and
-plans that share them give what each gives alone."""
+plans that share them give what each gives alone; they have the priority of the stream they serve."""
 
 import numpy as np
 import pytest
@@ -67,3 +67,16 @@ def test_resident_plans_of_a_server_share_side_streams():
     assert len(ctx.side_streams()) <= 7 * slots
     srv.close()
     assert ctx.side_streams() == []
+
+
+def test_side_streams_have_the_priority_of_the_program_s_stream():
+    torch = pytest.importorskip("torch")
+    streams = [torch.cuda.Stream(priority=p) for p in torch.cuda.Stream.priority_range()]
+    assert streams[0].priority != streams[1].priority
+    for stream in streams:
+        ctx = _context(stream.cuda_stream)
+        b = _batch(ctx, _problems(1))
+        b.run()
+        assert (b.sync() == 0).all()
+        got = [torch.cuda.ExternalStream(s).priority for s in ctx.side_streams()]
+        assert got and set(got) == {stream.priority}
