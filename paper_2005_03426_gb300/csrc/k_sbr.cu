@@ -95,7 +95,12 @@ __device__ __forceinline__ double2 sbr_sub(double2 a, double2 f, double2 v) { re
 // Shared memory of one group.  B and D: the step's two blocks, column-major with a padded column
 // (LD even: two rows of a column are one aligned 16-byte read, and consecutive columns fall in
 // other banks).
-template <class C, int BMAX, int P>
+template <class C, int BMAX, bool EARLY> struct SbrLate {};
+template <class C, int BMAX> struct SbrLate<C, BMAX, true> {
+    C dl[BMAX];          // D's last row and B's last entry, taken from the predecessor's published row
+    C bl, d00;
+};
+template <class C, int BMAX, int P, bool EARLY>
 struct __align__(16) SbrGroup {
     static constexpr int LD = BMAX + 2;
     typedef typename SbrDup<C>::T Dup;
@@ -106,9 +111,11 @@ struct __align__(16) SbrGroup {
     C red[3][P][BMAX];   // partial sums: B v_p, v^H B, D v
     C c0[BMAX];          // B(:, 0)
     C ty[BMAX];
-    C dl[BMAX];          // D's last row and B's last entry, taken from the predecessor's published row
-    C bl, beta, d00, pad;
+    C beta, pad;
+    SbrLate<C, BMAX, EARLY> late;
 };
+
+__host__ __device__ constexpr bool sbr_early(int cl, int ng) { return cl >= 4 || ng >= 8; }
 
 // Predicated load (zero where !ok) and store of one complex element, without a branch around each.
 // CG reads L2 only: the CTAs of a cluster run on different SMs, whose L1 caches are not coherent, so
@@ -211,15 +218,17 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
 // step's vectors are known, so a sweep follows its predecessor by a step and the part of a step up to
 // there, with its loads and B v_p done beforehand, where it waited for two whole steps (one FP32 system
 // of n = 1323 15.1 -> 13.2 ms, eight in FP64 99 -> 87).  With few groups per system (CL <= 2 and wide
-// windows) the SMs are busy anyway (64 systems: 25.0 ms with the publication, 25.2 without): there a sweep
-// waits for all of the predecessor's step s + 1.
+// windows) the SMs are busy anyway (64 systems: 24.9 ms with the publication, 23.7 without): there a sweep
+// waits for all of the predecessor's step s + 1, and the publication's code, its shared memory and its
+// terms in the stores' conditions are compiled out (left to run-time conditions that are constant they cost
+// 64 systems 1 %).
 //
 // What bounds it: the critical path of one sweep after another (about 1.5 n steps), so the latency of a
 // step; on the FP64 path the 2 FP64 FMAs per clock
 // of an SM (24 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
 // CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
 // b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
-// kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 25.2 ms; eight systems in FP64
+// kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
 // 455 -> 87 ms.
 //
 // CL = 1: one CTA per system.  CL > 1: a cluster of CL CTAs per system, the sweeps dealt round-robin
@@ -236,13 +245,13 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                                                           double* __restrict__ dvec, double* __restrict__ evec,
                                                           int* __restrict__ status) {
     typedef typename Cx<R>::T C;
-    typedef SbrGroup<C, BMAX, P> Grp;
+    constexpr bool EARLY = sbr_early(CL, NG);       // first rows published ahead
+    typedef SbrGroup<C, BMAX, P, EARLY> Grp;
     typedef SbrDup<C> DupC;
     constexpr int G = BMAX * P, EL = BMAX / P, LD = Grp::LD;
     constexpr int SL = BMAX >= 32 ? BMAX / 32 : 1;  // entries of a vector per lane
     constexpr bool F64 = sizeof(R) == 8;            // FP64 units are scarce: skip padding
     constexpr int NGT = CL * NG;                    // groups per system
-    constexpr bool EARLY = CL >= 4 || NG >= 8;      // first rows published ahead
     static_assert(G % 32 == 0 && EL * P == BMAX && EL % 2 == 0, "group shape");
     extern __shared__ __align__(16) unsigned char sbr_smem[];
     long long* key = reinterpret_cast<long long*>(sbr_smem);
@@ -286,9 +295,9 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
     int cur = 0;  // buffer of the current reflector in S.v
     bool stopped = false;
     C tau = zero, taup = zero;
-    // a warp's bounded wait for a predecessor's progress (acquire); after one gave up nobody waits
+    // a warp's bounded wait for a predecessor's progress (acquire); after one gave up nobody waits (the
+    // caller asks: an early return in here costs a spilled flag in every step, 64 systems 25.6 ms for 23.9)
     auto wait_for = [&](uint32_t where, long long need) {
-        if (stopped) return;
         if (lane == 0) {
             int it = 0;
             while (key_load(where) < need) {
@@ -311,7 +320,8 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             // rows r .. r + b - 2 are the predecessor's of its step s, which it has to have finished;
             // row r + b - 1, if there is one, is the first row of its step s + 1, published during it
             // (without publication: all of step s + 1)
-            if (j > 0) wait_for(pkey, (long long)(j - 1) * KK + (EARLY ? s + 1 : s + 2 < KK - 1 ? s + 2 : KK - 1));
+            if (j > 0 && !stopped)
+                wait_for(pkey, (long long)(j - 1) * KK + (EARLY ? s + 1 : s + 2 < KK - 1 ? s + 2 : KK - 1));
             const int r = j + 1 + s * b, rp = r - b;
             const int l = min(b, n - r);
             const bool late = EARLY && j > 0 && l == b;
@@ -338,7 +348,9 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             }
 #pragma unroll
             for (int q = 0; q < EL; ++q) S.D[(k0 + q) * LD + i] = i == k0 + q ? zero : D[q];
-            if (tid == 0) S.d00 = D[0];
+            if constexpr (EARLY) {
+                if (tid == 0) S.late.d00 = D[0];
+            }
             if (s > 0) {
                 // y = B v_p over this thread's columns
                 const auto* vp = S.v[cur ^ 1] + k0;
@@ -364,20 +376,20 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             if (warp == 0) {
                 R part = R(0);
                 C bl = zero;  // B(b-1, b-1), the only nonzero of B's last row; at s = 0 x(b-1)
-                if (late) {
-                    wait_for(ppub, (long long)(j - 1) * KK + (s + 2));
+                if constexpr (EARLY) if (late) {
+                    if (!stopped) wait_for(ppub, (long long)(j - 1) * KK + (s + 2));
                     const C* h = Hg + r + b - 1;
                     bl = ld_if<(CL > 1)>(h + (r - 1) * ldi, true);
 #pragma unroll
                     for (int u = 0; u < SL; ++u) {
                         const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
                         const C dl = ld_if<(CL > 1)>(h + (r + (e < b ? e : 0)) * ldi, e < b);
-                        S.dl[e] = dl;
+                        S.late.dl[e] = dl;
                         if (e < b - 1) S.D[e * LD + b - 1] = dl;
                         if (s == 0 && e == b - 1) x[u] = bl;
                     }
                     if (lane == 0) {
-                        S.bl = bl;
+                        S.late.bl = bl;
                         if (s > 0) S.B[(b - 1) * LD + b - 1] = bl;
                     }
                 }
@@ -389,9 +401,11 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
 #pragma unroll
                         for (int q = 1; q < P; ++q) y = y + S.red[0][q][e];
                         C c0 = S.c0[e];
-                        if (late && e == b - 1) {
-                            y = y + bl * DupC::val(S.v[cur ^ 1][b - 1]);
-                            if (b == 1) c0 = bl;
+                        if constexpr (EARLY) {
+                            if (late && e == b - 1) {
+                                y = y + bl * DupC::val(S.v[cur ^ 1][b - 1]);
+                                if (b == 1) c0 = bl;
+                            }
                         }
                         ty[u] = taup * y;
                         x[u] = c0 - ty[u];   // v_p[0] = 1
@@ -415,11 +429,11 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             }
             gbar<G>(g);
             const auto* v = S.v[cur];
-            if (late && i == b - 1) {  // the owners of the last row
+            if constexpr (EARLY) if (late && i == b - 1) {  // the owners of the last row
 #pragma unroll
                 for (int q = 0; q < EL; ++q) {
-                    if (k0 + q < b) D[q] = S.dl[k0 + q];
-                    if (s > 0 && k0 + q == b - 1) B[q] = S.bl;
+                    if (k0 + q < b) D[q] = S.late.dl[k0 + q];
+                    if (s > 0 && k0 + q == b - 1) B[q] = S.late.bl;
                 }
             }
             // (c) column i over rows k0 .. k0 + EL - 1 of B and of D's strict lower triangle, and row i
@@ -490,7 +504,7 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             gbar<G>(g);
             // the first row of both blocks, published at once for the successor, whose step s - 1 has it
             // as its last row
-            if (EARLY && warp == G / 32 - 1) {
+            if constexpr (EARLY) if (warp == G / 32 - 1) {
                 const auto* vp = S.v[cur ^ 1];
 #pragma unroll
                 for (int u = 0; u < SL; ++u) {
@@ -503,7 +517,7 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                 }
                 if (lane == 0) {
                     const C w0 = DupC::val(S.wd[0]);
-                    C a = late && b == 1 ? S.dl[0] : S.d00;
+                    C a = late && b == 1 ? S.late.dl[0] : S.late.d00;
                     a = mk(a.x - R(2) * w0.x, R(0));  // v_0 = 1
                     st_if(Hg + r * ldi + r, a, true);
                     if (s == 0) {
@@ -516,7 +530,6 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
             }
             // (e) rank-2 updates of this thread's other entries, back to global memory
             const C vi = DupC::val(v[i]), wi = DupC::val(S.wd[i]);
-            const bool st = (!EARLY || i > 0) && i < l;
             if (s > 0) {
                 const C tyi = S.ty[i];
                 const auto *vp = S.v[cur ^ 1] + k0, *wu = S.wu + k0;
@@ -526,7 +539,8 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                     if (F64 && k0 + q >= b) continue;
                     C a = sbr_sub(sbr_sub_conj(B[q], tyi, vp[q]), vi, wu[q]);
                     if (q == 0 && p == 0) a = i == 0 ? S.beta : zero;
-                    st_if(h + q * ldi, a, st && k0 + q < b);
+                    if constexpr (EARLY) st_if(h + q * ldi, a, i > 0 && i < l && k0 + q < b);
+                    else st_if(h + q * ldi, a, i < l && k0 + q < b);
                 }
             }
             if (row) {
@@ -539,7 +553,8 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
                     // v_i conj(w_k) + w_i conj(v_k)
                     C a = sbr_sub_conj(sbr_sub_conj(D[q], vi, wd[q]), wi, vk[q]);
                     if (i == k) a.y = R(0);
-                    st_if(h + q * ldi, a, st && i >= k);
+                    if constexpr (EARLY) st_if(h + q * ldi, a, i > 0 && i < l && i >= k);
+                    else st_if(h + q * ldi, a, i >= k && i < l);
                     if (!EARLY && q == 0 && s == 0 && tid == 0) dd[j + 1] = (double)a.x;
                 }
             }
@@ -548,12 +563,9 @@ __global__ void __launch_bounds__(BMAX* P* NG) k_sbr_chase(const MmfDesc* __rest
 #pragma unroll
                     for (int u = 0; u < SL; ++u) {
                         const int e = BMAX >= 32 ? lane + 32 * u : lane % BMAX;
-                        if (e > 0 && e < l) Hg[j * ldi + r + e] = zero;
-                        if (!EARLY && e == 0 && lane == 0) {
-                            Hg[j * ldi + r] = mk(beta, R(0));
-                            ee[j] = (double)beta;
-                        }
+                        if (EARLY ? e > 0 && e < l : e < l) Hg[j * ldi + r + e] = e == 0 ? mk(beta, R(0)) : zero;
                     }
+                    if (!EARLY && lane == 0) ee[j] = (double)beta;
                 }
                 // store the reflector for the back-transform, marked evict-first: the store is
                 // written once and read only after the chase, and L2 should keep the band's lines
@@ -794,8 +806,8 @@ template <class R, int BMAX, int P, int NG, int CL>
 static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
                                    int* status, bool* fits) {
     typedef typename Cx<R>::T C;
-    static_assert(sizeof(SbrGroup<C, BMAX, P>) % 16 == 0, "group blocks keep 16-byte alignment");
-    const size_t sm = sbr_hdr(NG) + sizeof(SbrGroup<C, BMAX, P>) * NG;
+    static_assert(sizeof(SbrGroup<C, BMAX, P, sbr_early(CL, NG)>) % 16 == 0, "group blocks keep 16-byte alignment");
+    const size_t sm = sbr_hdr(NG) + sizeof(SbrGroup<C, BMAX, P, sbr_early(CL, NG)>) * NG;
     auto kern = k_sbr_chase<R, BMAX, P, NG, CL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -822,7 +834,7 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
 
 // The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
 // pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
-// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 25 ms that 64 such systems
+// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
 // take, with 8 it takes 13.2.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
