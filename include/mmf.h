@@ -390,6 +390,10 @@ MMF_API int mmf_selftest_split_tf32(int M, int N, int K, int mode, double* max_r
  * B = Q^H A Q, and returns max |B - tridiag(e, d, e)| over all entries and max |A|.  Allocates its
  * own device memory; for health checks, not for the solve path. */
 MMF_API int mmf_selftest_hetrd(int n, int count, int tensor_cores, double* max_abs_err, double* max_abs_ref);
+/* The thread-block cluster size (1, 2, 4, 6 or 8 CTAs per system) with which the dense reduction of a
+ * batch runs on the current device: `count` systems on it, the largest of dimension n (above the
+ * one-CTA kernel's 103 in FP64 and 152 in mixed precision, and not of the whole-GPU path). */
+MMF_API int mmf_selftest_hetrd_ctas(int n, int count, int precision, int tensor_cores, int* ctas);
 
 /* ---------------------------------------------------------------- misc */
 MMF_API const char* mmf_strerror(int status);

@@ -34,6 +34,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "mmf_internal.h"
@@ -831,8 +832,9 @@ int mmf_hetrd_max_n(int fp32) {
 // CL CTAs per system; *fits (if given) only reports whether one wave holds all the clusters.
 template <class R, int CL, bool TC>
 static cudaError_t launch_hetrd_cl(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
-                                   double* evec, void* tau, size_t sm, int* status, bool* fits) {
+                                   double* evec, void* tau, int* status, bool* fits) {
     typedef typename Cx<R>::T C;
+    const size_t sm = hetrd_smem(L.nmax, sizeof(R) == 4);
     cudaError_t err = cudaFuncSetAttribute(k_hetrd<R, CL, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
@@ -859,41 +861,52 @@ static cudaError_t launch_hetrd_cl(const MmfLaunch& L, void* H, void* Vp, void* 
 
 // The most CTAs per system that run in one wave (a GB300 holds 15 clusters of 8, 23 of 6, 36 of 4);
 // from 4 on only for systems long enough that each CTA keeps a few row chunks (the barriers of a larger
-// cluster cost more than a small column's work).
+// cluster cost more than a small column's work).  *ctas (if given) only reports the choice.
 template <class R, bool TC>
 static cudaError_t launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
-                                double* evec, void* tau, size_t sm, int* status) {
-    bool fits = false;
-    cudaError_t e;
+                                double* evec, void* tau, int* status, int* ctas) {
+    cudaError_t e = cudaSuccess;
+    bool done = false;
+    auto attempt = [&](auto cl) {  // taken if its clusters fit one wave, and at the latest with one CTA per system
+        constexpr int CL = decltype(cl)::value;
+        if (done || e != cudaSuccess) return;
+        bool fits = CL == 1;
+        if (!fits) e = launch_hetrd_cl<R, CL, TC>(L, H, Vp, Wp, dvec, evec, tau, status, &fits);
+        if (e != cudaSuccess || !fits) return;
+        done = true;
+        if (ctas) *ctas = CL;
+        else e = launch_hetrd_cl<R, CL, TC>(L, H, Vp, Wp, dvec, evec, tau, status, nullptr);
+    };
     if (L.nmax >= HT_CL8_N) {
-        e = launch_hetrd_cl<R, 8, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
-        if (e != cudaSuccess) return e;
-        if (fits) return launch_hetrd_cl<R, 8, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+        attempt(std::integral_constant<int, 8>());
+        attempt(std::integral_constant<int, 6>());
     }
-    if (L.nmax >= HT_CL8_N) {
-        e = launch_hetrd_cl<R, 6, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
-        if (e != cudaSuccess) return e;
-        if (fits) return launch_hetrd_cl<R, 6, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
-    }
-    if (L.nmax >= HT_CL4_N) {
-        e = launch_hetrd_cl<R, 4, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
-        if (e != cudaSuccess) return e;
-        if (fits) return launch_hetrd_cl<R, 4, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
-    }
-    e = launch_hetrd_cl<R, 2, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, &fits);
-    if (e != cudaSuccess) return e;
-    if (fits) return launch_hetrd_cl<R, 2, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
-    return launch_hetrd_cl<R, 1, TC>(L, H, Vp, Wp, dvec, evec, tau, sm, status, nullptr);
+    if (L.nmax >= HT_CL4_N) attempt(std::integral_constant<int, 4>());
+    attempt(std::integral_constant<int, 2>());
+    attempt(std::integral_constant<int, 1>());
+    return e;
+}
+
+static cudaError_t hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec, double* evec, void* tau,
+                         int fp32, int tc, int* status, int* ctas) {
+    if (L.nmax > mmf_hetrd_max_n(fp32)) return cudaErrorInvalidValue;
+    if (fp32 && tc) return launch_hetrd<float, true>(L, H, Vp, Wp, dvec, evec, tau, status, ctas);
+    if (fp32) return launch_hetrd<float, false>(L, H, Vp, Wp, dvec, evec, tau, status, ctas);
+    return launch_hetrd<double, false>(L, H, Vp, Wp, dvec, evec, tau, status, ctas);
 }
 
 cudaError_t mmf_launch_hetrd(const MmfLaunch& L, void* H, void* Vp, void* Wp, double* dvec,
                              double* evec, void* tau, int fp32, int tc, int* status) {
     if (L.count <= 0) return cudaSuccess;
-    if (L.nmax > mmf_hetrd_max_n(fp32)) return cudaErrorInvalidValue;
-    const size_t sm = hetrd_smem(L.nmax, fp32);
-    if (fp32 && tc) return launch_hetrd<float, true>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
-    if (fp32) return launch_hetrd<float, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
-    return launch_hetrd<double, false>(L, H, Vp, Wp, dvec, evec, tau, sm, status);
+    return hetrd(L, H, Vp, Wp, dvec, evec, tau, fp32, tc, status, nullptr);
+}
+
+// CTAs per system that a launch of `count` systems, the largest of dimension n, takes
+cudaError_t mmf_hetrd_ctas(int n, int count, int fp32, int tc, int* ctas) {
+    MmfLaunch L = {};
+    L.count = count;
+    L.nmax = n;
+    return hetrd(L, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, fp32, tc, nullptr, ctas);
 }
 
 // ------------------------------------------------------------------ self-test

@@ -2318,6 +2318,15 @@ extern "C" int mmf_selftest_hetrd(int n, int count, int tensor_cores, double* ma
     return MMF_OK;
 }
 
+extern "C" int mmf_selftest_hetrd_ctas(int n, int count, int precision, int tensor_cores, int* ctas) {
+    const int fp32 = precision == MMF_MIXED;
+    if (!ctas || (precision != MMF_FP64 && !fp32)) return fail(MMF_ERR_ARG, "precision and ctas required");
+    if (count < 1 || n <= mmf_hetrd_small_n(fp32) || n > mmf_hetrd_max_n(fp32))
+        return fail(MMF_ERR_ARG, "no size of the cluster reduction");
+    CU(mmf_hetrd_ctas(n, count, fp32, tensor_cores, ctas));
+    return MMF_OK;
+}
+
 extern "C" int mmf_selftest_gram(int n, double* max_abs_err, double* max_abs_ref) {
     if (!max_abs_err || !max_abs_ref) return fail(MMF_ERR_ARG, "output pointers required");
     int rc = mmf_ozaki_selftest_impl(n, max_abs_err, max_abs_ref);

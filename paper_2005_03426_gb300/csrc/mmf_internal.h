@@ -277,6 +277,7 @@ cudaError_t mmf_launch_outputs(const MmfLaunch& L, int Mmax, int Dmax, const dou
                                const double2* Z, float2* Z1, float2* Zlo, const double* t, double t0, int nt,
                                double2* F, double2* U, double* P, double cluster_rel, int skip_u, int skip_p,
                                void* scratch, int scratch_esz);
+cudaError_t mmf_hetrd_ctas(int n, int count, int fp32, int tc, int* ctas);
 int mmf_hetrd_max_n(int fp32);
 // the same reduction with the whole matrix in one CTA's shared memory (k_hetrd_small.cu), for n up to
 // mmf_hetrd_small_n

@@ -140,6 +140,7 @@ _SIGS = {
     "mmf_selftest_gram": (_I, [_I, ctypes.POINTER(_D), ctypes.POINTER(_D)]),
     "mmf_selftest_split_tf32": (_I, [_I, _I, _I, _I, ctypes.POINTER(_D), ctypes.POINTER(_D)]),
     "mmf_selftest_hetrd": (_I, [_I, _I, _I, ctypes.POINTER(_D), ctypes.POINTER(_D)]),
+    "mmf_selftest_hetrd_ctas": (_I, [_I, _I, _I, _I, ctypes.POINTER(_I)]),
     "mmf_strerror": (ctypes.c_char_p, [_I]),
     "mmf_spin_components": (_I, [_I, _P, _P, _I, _P]),
     "mmf_last_error": (ctypes.c_char_p, []),
