@@ -528,5 +528,3 @@ cudaError_t mmf_launch_hetrd_large(const MmfDesc& d, void* H, void* Vp, void* Wp
                              (double2*)work, (LgScalars*)sc, dvec + d.vec_off, evec + d.vec_off,
                              (double2*)tau + d.vec_off, st);
 }
-
-size_t mmf_hetrd_large_scalars_bytes() { return sizeof(LgScalars); }
