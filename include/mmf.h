@@ -104,7 +104,8 @@ MMF_API int mmf_ctx_side_streams(mmf_ctx* ctx, void** streams, int cap);
  * mmf_batch_sync / mmf_diagonalise.
  * MMF_OPT_HETRD_TC: in the mixed path, the dense Householder reduction's trailing update
  * A -= V W^H + W V^H after each panel (Sec. 3.2's diagonalisation) on the tensor cores in split
- * TF32 (1 or < 0, default) or on the FP32 units (0).
+ * TF32 (1 or < 0, default) or on the FP32 units (0).  Systems of n <= 152 are reduced column by column
+ * in one CTA's shared memory, on the FP32 units whatever the option says.
  * Results do not depend on the path beyond rounding. */
 #define MMF_OPT_JACOBI_N_FP64 1
 #define MMF_OPT_JACOBI_N_MIXED 2
@@ -384,7 +385,7 @@ MMF_API int mmf_selftest_split_tf32(int M, int N, int K, int mode, double* max_r
                                     double* max_rel_err_fp32);
 /* Runs the mixed path's FP32 Householder reduction to tridiagonal form (Sec. 3.2's
  * diagonalisation, first step) on `count` seeded Hermitian n x n FP32 matrices in one launch
- * (2 <= n <= the one-CTA maximum, count <= 512, n^2 count <= 2^27), with the trailing update
+ * (2 <= n <= the cluster reduction's maximum, count <= 512, n^2 count <= 2^27), with the trailing update
  * A -= V W^H + W V^H on the tensor cores in split TF32 (tensor_cores = 1) or on the FP32 units
  * (0).  For the first two matrices the host applies the stored reflectors in FP64,
  * B = Q^H A Q, and returns max |B - tridiag(e, d, e)| over all entries and max |A|.  Allocates its

@@ -17,10 +17,10 @@
 // Result: d (diagonal), e = beta (sub-diagonal, real), tau, and v[k+2:] stored in
 // A(k+2:, k).  Q = P_0 P_1 ... P_{n-2}, Q^H H_F Q = tridiag(e, d, e).
 //
-// One thread-block cluster of CL CTAs (512 threads each, CL = 1, 2, 4 or 8) per system.  The hemv
+// One thread-block cluster of CL CTAs (512 threads each, CL = 1, 2, 4, 6 or 8) per system.  The hemv
 // streams the lower triangle of the trailing matrix once per column with coalesced column reads: a
-// warp owns 8 columns, lanes own rows, the row part accumulates through shared-memory atomics and
-// the column part by warp-shuffle reductions.  The CTAs split the column blocks of the hemv and the
+// warp takes tasks of rows (dealt over its lanes) x columns, sums the row part in registers and the
+// column part by an exchange over the lanes, and adds both to y in shared memory.  The CTAs split the column blocks of the hemv and the
 // tiles of the trailing update; everything of length m is split by rows (chunks of 32 rows dealt
 // round-robin): the pending panel updates of the column, the dot products W^H v and V^H v, and the
 // corrections of y.  Per column three cluster barriers: the column and its norm reach every CTA
@@ -450,7 +450,7 @@ k_hetrd(const MmfDesc* __restrict__ descs, const int* __restrict__ idx,
     R* nrmP = red + 16;                         // by the partners: parts of ||x||^2 (8),
     R* dotP = red + 49;                         // parts of w^H v (8 complex),
     R* wnxt = red + 66;                         // w at row k + 1 before its last correction (complex)
-    // one region shared by the her2k staging tiles and (FP32) the hemv's cp.async stages
+    // one region shared by the partial sums of the O(m i) steps and the trailing update's operands
     C* big = reinterpret_cast<C*>(smem_raw + ht_big_offset<R>(nmax));
     C* tVr = big;                               // MMF_NB x HT_TILE (her2k staging, transposed)
     C* tWr = tVr + MMF_NB * HT_TILE;
@@ -910,8 +910,8 @@ cudaError_t mmf_hetrd_ctas(int n, int count, int fp32, int tc, int* ctas) {
 
 // ------------------------------------------------------------------ self-test
 // `count` seeded Hermitian n x n FP32 matrices (entries uniform in the unit square, full
-// mantissas; leading dimension n rounded up to 8) reduced in one launch (two CTAs per system when
-// 2 count fits the SMs, else one), with the trailing update on the tensor cores (tc = 1) or the
+// mantissas; leading dimension n rounded up to 8) reduced in one launch (at any n, also where a plan
+// takes the one-CTA kernel), with the trailing update on the tensor cores (tc = 1) or the
 // FP32 units (tc = 0).  For the first two systems the host applies the stored reflectors to the
 // input in FP64, B = P_{n-2}^H ... P_0^H A P_0 ... P_{n-2}, and returns max |B - tridiag(e, d, e)|
 // (every entry) and max |A|.  Returns 0, -1 (bad sizes), -4 (CUDA failure) or 1 (a wait gave up).

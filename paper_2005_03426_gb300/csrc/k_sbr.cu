@@ -16,9 +16,10 @@
 // All reflectors satisfy H^H x = beta e_1 with beta real (H = I - tau v v^H, v[0] = 1; the
 // convention of k_hetrd), so T = Q^H H_F Q is real and Q = prod_j prod_s H(j, s).
 //
-// Pipelining: sweep j+1 may run its step s once sweep j has finished step s+1 (their later
-// steps touch disjoint entries), so several sweeps are in flight at once, each with a group of
-// threads of its own that publishes its progress and waits (bounded) for its predecessor's.  The
+// Pipelining: sweep j+1 may run its step s once sweep j has finished step s and the first row of
+// its step s+1 (their later steps touch disjoint entries), so several sweeps are in flight at once,
+// each with a group of threads of its own that publishes its progress and waits (bounded) for its
+// predecessor's.  The
 // band itself stays in the dense matrix's lower triangle (global memory, L2-resident: about n x 2b
 // entries are ever touched).
 //
@@ -226,7 +227,7 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
 // What bounds it: the critical path of one sweep after another (about 1.5 n steps), so the latency of a
 // step; on the FP64 path the 2 FP64 FMAs per clock
 // of an SM (24 b^2 FMAs a step).  NG groups per CTA and CL CTAs (SMs) per system hold
-// CL x NG sweeps in flight; more than n / (2 b) of them have nothing to do.  Measured at n = 1323,
+// CL x NG sweeps in flight (how many have work: see launch_chase).  Measured at n = 1323,
 // b = 63 (128 threads per sweep with both blocks in shared memory, at most two CTAs per system -> this
 // kernel): one system in FP32 36.2 -> 13.2 ms, 64 systems 37.4 -> 23.7 ms; eight systems in FP64
 // 455 -> 87 ms.
@@ -832,14 +833,16 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
     return cudaLaunchKernelEx(&cfg, kern, L.desc, L.idx, (C*)H, (C*)store, dvec, evec, status);
 }
 
-// The most CTAs per system (1, 2, 4 or 8) that run in one wave, and no more than give the
-// pipeline work: sweeps start two steps apart, so about n / (2 b) of them are in flight.  One
-// system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that 64 such systems
-// take, with 8 it takes 13.2.
+// The most CTAs per system (1, 2, 4 or 8) that run in one wave, doubled while the sweeps in flight
+// exceed the groups of half of them.  A sweep has up to n / b steps and starts two steps behind its
+// predecessor, about one and a half where first rows are published ahead: n / (2 b) to n / (1.5 b) in
+// flight, for which the rule takes n / BMAX (b lies in the upper half of a window class, but anywhere in
+// the smallest one).  One system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that
+// 64 such systems take, with 8 it takes 13.2.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
                                 int* status) {
-    const int sweeps = L.nmax / BMAX + 1;  // b > BMAX / 2, so at least n / (2 b)
+    const int sweeps = L.nmax / BMAX + 1;
     bool fits = false;
     cudaError_t e = cudaSuccess;
     if (sweeps > 4 * NG) {
