@@ -29,7 +29,9 @@
 //
 // What bounds it: with one system per two SMs the hemv's L2 reads and the 2i column reads of the
 // panel, repeated by each CTA; with 8 SMs a system the barriers and L2 latencies of a column (a few
-// microseconds), which is why the split reaches the O(m i) steps too.
+// microseconds), which is why the split reaches the O(m i) steps too.  Two systems of n = 1792 in FP32 on 8
+// SMs each: 40 ms, of 10.9 warp cycles per instruction 3.2 wait at barriers and 1.4 for loads, L2 at 2 % of
+// its rate.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -124,7 +126,7 @@ __device__ __forceinline__ void atomic_add_c(float2* p, float2 v) {
 // the task; the column parts of a block are summed over the lanes by one butterfly that halves the
 // values at each exchange.  A warp's time is the latency of its chain
 // of loads and exchanges (L2 latency near 1000 cycles), so few long steps beat many short ones: at
-// m = 1000 on 8 SMs 9 us, 27 bytes a clock and SM, where blocks of 4 columns with an exchange and two
+// m = 1000 on 8 SMs 9 us, 27 bytes a clock and SM (this product alone, in a loop), where blocks of 4 columns with an exchange and two
 // in flight take 12; a ring of cp.async pieces 7 columns deep takes 15 (its instructions per column).
 // (HT_NL = 8 measures the same and needs more registers.)  cw is chosen so that every warp gets a few
 // tasks.

@@ -8,8 +8,9 @@
 // The lower triangle is kept packed by columns (n (n + 1) / 2 entries), so several CTAs share an SM.
 //
 // Why a kernel of its own: at n = 82 the panel form of k_hetrd spends a column's 50 microseconds in
-// barriers, L2 latencies and short dot products over the panel.  Here the FP64 units bound it (one
-// warp-wide FP64 instruction per 64 cycles and scheduler, 19 cycles over the SM's four): the O(m^2)
+// barriers, L2 latencies and short dot products over the panel.  Here the FP64 units are what a column
+// waits for most (one warp-wide FP64 instruction per 64 cycles and scheduler, 19 cycles over the SM's four:
+// one system keeps its SM's at 61 %, the rest is barriers and shared memory's latency): the O(m^2)
 // steps run on all warps (the update over the packed triangle's entries in line, so that no lane idles
 // at a column's end), the O(m) ones a row per thread, and the scalars in one warp.  Measured in FP64
 // at n = 82: one system 1.0 ms (k_hetrd 4.3), 200 systems 1.5 ms (k_hetrd 8.4).
@@ -143,10 +144,10 @@ k_hetrd_small(const MmfDesc* __restrict__ descs, const int* __restrict__ idx, ty
 
 // Back-transform Z = P_0 P_1 ... P_{n-2} Y of the same systems (S5): a CTA takes HS_BT_NC columns of
 // Z in shared memory and applies the reflectors one by one, last first, each column's rows dealt over
-// HS_BT_RG threads.  FP64-bound like the reduction (8 n^3 / 2 real flops a system), with two barriers a
-// reflector, where the blocked form's T factors and 64-row tiles cost more than they save at these
-// sizes: n = 82 in FP64, one system 0.27 ms (k_larft and k_backtransform 1.27), 200 systems 1.2 ms
-// (4.65).
+// HS_BT_RG threads.  Bound by the FP64 units (8 n^3 / 2 real flops a system; 93 % of their rate with 200
+// systems), with two barriers a reflector, where the blocked form's T factors and 64-row tiles cost more
+// than they save at these sizes: n = 82 in FP64, one system 0.2 ms (k_larft and k_backtransform 1.27), 200
+// systems 1.2 ms (4.65).
 #define HS_BT_NC 16
 #define HS_BT_THREADS 128
 #define HS_BT_RG (HS_BT_THREADS / HS_BT_NC)

@@ -837,7 +837,9 @@ static cudaError_t launch_chase_cl(const MmfLaunch& L, void* H, double2* store, 
 // exceed the groups of half of them.  A sweep has up to n / b steps and starts two steps behind its
 // predecessor, about one and a half where first rows are published ahead: n / (2 b) to n / (1.5 b) in
 // flight, for which the rule takes n / BMAX (b lies in the upper half of a window class, but anywhere in
-// the smallest one).  One system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that
+// the smallest one).  Twice that estimate gives the same times within 1 % from b = 7 to 63, n = 244 to 800,
+// 1 to 12 systems, in both precisions; b = 3 at n = 242 would be 10 % (FP32) or 12 % (FP64) faster with the
+// 8 CTAs it then takes for 4.  One system of n = 1323, b = 63 in FP32 with 2 CTAs per system takes the 24 ms that
 // 64 such systems take, with 8 it takes 13.2.
 template <class R, int BMAX, int P, int NG>
 static cudaError_t launch_chase(const MmfLaunch& L, void* H, double2* store, double* dvec, double* evec,
